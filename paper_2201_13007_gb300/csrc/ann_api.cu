@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "ann_internal.cuh"
+#include "knn.cuh"
 
 struct ann_index {
     ann::IndexData d;
@@ -545,21 +546,20 @@ int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, in
         return fail(ANN_ERR_ARG, "self_offset=%lld does not place the queries inside the base", (long long)self_offset);
     if (nq == 0) return ANN_OK;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    float *norms = nullptr;
-    int *err = nullptr;
+    const int sms = sm_count();
+    const ann::KnnPlan plan = ann::knn_plan(n, nq, sms);
+    unsigned char *ws = nullptr;
     cudaError_t e;
-    if ((e = cudaMalloc(&norms, (size_t)ann::knn_norms_rows(n) * 4 + 16)) != cudaSuccess)
-        return cuda_fail(e, "cudaMalloc(knn norms)");
-    err = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(norms) + (size_t)ann::knn_norms_rows(n) * 4);
+    if ((e = cudaMalloc(&ws, plan.bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc(knn workspace)");
     int herr = 0;
-    if ((e = cudaMemsetAsync(err, 0, 4, s)) == cudaSuccess &&
-        (e = ann::launch_knn_bf16(base, n, d, queries, nq, self_offset, metric, k, out_ids, out_dists, norms, err,
+    if ((e = ann::launch_knn_bf16(plan, ws, base, n, d, queries, nq, self_offset, metric, k, out_ids, out_dists, sms,
                                   s)) == cudaSuccess &&
-        (e = cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
+        (e = cudaMemcpyAsync(&herr, ws + plan.err, 4, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
         e = cudaStreamSynchronize(s);
-    cudaFree(norms);
+    if (e != cudaSuccess) cudaStreamSynchronize(s);  // nothing may use the workspace when it is freed
+    cudaFree(ws);
     if (e != cudaSuccess) return cuda_fail(e, "knn");
-    if (herr) return fail(ANN_ERR_CUDA, "knn: a candidate merge did not converge");
+    if (herr) return fail(ANN_ERR_CUDA, "knn: a %s did not end", herr == 2 ? "wait" : "candidate merge");
     return ANN_OK;
 }
 

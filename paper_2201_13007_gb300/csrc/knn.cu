@@ -3,6 +3,11 @@
 // Sec. 2.2 builds on proximity graphs such as NSG and HNSW; its k-NN
 // candidate lists are the exact Def. 1 neighbours of every base point).
 //
+// This is the scan: exact keys from the first tile on, whatever the data. Since
+// the filter of knn_filter.cu it runs only for the blocks of 128 query rows that
+// the filter hands over (a list that ran over, values it cannot bound); its keys
+// define the result of both.
+//
 // The distance matrix of a brute-force scan is n x n (10^14 entries at 10M
 // points), so it must never reach HBM: each CTA holds 128 query rows as
 // tensor-core operands in registers, streams the whole base set through
@@ -17,54 +22,15 @@
 // BF16 x BF16 products are exact in FP32; sums are FP32. Keys are the FP32
 // distance (squared l2, or -<q, x>) under an order-preserving map to
 // unsigned, so (key, id) sorts like (distance, id).
-#include <cuda_bf16.h>
-
-#include "ann_internal.cuh"
+#include "knn_common.cuh"
 
 namespace ann {
 namespace {
 
-constexpr int KBM = 128;    // query rows per CTA
 constexpr int KBN = 128;    // base rows per tile
 constexpr int KLIST = 64;   // list length per query row
 constexpr int KCAP = 32;    // candidate buffer per query row
 constexpr int KNT = 256;    // 8 warps: 4 along the query rows x 2 along the tile's base rows
-constexpr unsigned long long KMAX = ~0ull;
-
-__device__ __forceinline__ uint32_t ord_enc(float f) {
-    const uint32_t b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-__device__ __forceinline__ float ord_dec(uint32_t u) {
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u);
-}
-
-__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-        "{%0,%1,%2,%3};\n"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Four 8x8 BF16 matrices; lane i names row i % 8 of matrix i / 8.
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], uint32_t saddr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(saddr));
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const void *gmem, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(saddr), "l"(gmem), "r"(valid ? 16 : 0)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 
 struct KnnSmem {
     unsigned long long *list;  // [KBM][KLIST], ascending
@@ -77,8 +43,6 @@ struct KnnSmem {
     int *cnt;                  // [KBM] appends since the last merge (may pass KCAP on overflow)
     int *flags;                // [0] overflow in the last pass, [1] merge rounds exhausted
 };
-
-__host__ __device__ constexpr int knn_pitch(int d) { return d + 8; }
 
 // Base tiles in flight: four while they fit beside the lists.
 __host__ __device__ constexpr int knn_stages(int d) { return d <= 96 ? 4 : 3; }
@@ -201,7 +165,9 @@ template <int KS, bool L2>
 __global__ void __launch_bounds__(KNT, 1)
     knn_bf16_kernel(const __nv_bfloat16 *__restrict__ base, const float *__restrict__ bnorm_g, int64_t n,
                     const __nv_bfloat16 *__restrict__ queries, int64_t nq, int64_t self0, int k,
-                    int32_t *__restrict__ out_ids, float *__restrict__ out_d, int *__restrict__ err) {
+                    int32_t *__restrict__ out_ids, float *__restrict__ out_d, const int *__restrict__ only,
+                    int *__restrict__ err) {
+    if (!only[blockIdx.x]) return;
     constexpr int D = KS * 16;
     constexpr int P = knn_pitch(D);
     constexpr int CPR = D / 8;  // 16-byte chunks per row
@@ -419,34 +385,17 @@ __global__ void __launch_bounds__(KNT, 1)
     }
 }
 
-// Squared norms of BF16 rows in FP32 (the same sum order as the kernel's
-// query norms), zero for the padding rows up to n_pad.
-__global__ void bf16_row_norms(const __nv_bfloat16 *__restrict__ x, int64_t n, int64_t n_pad, int d,
-                               float *__restrict__ out) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_pad) return;
-    float acc = 0.f;
-    if (r < n) {
-        const __nv_bfloat16 *p = x + r * d;
-        for (int i = 0; i < d; ++i) {
-            const float v = __bfloat162float(p[i]);
-            acc = fmaf(v, v, acc);
-        }
-    }
-    out[r] = acc;
-}
-
 template <int KS, bool L2>
 cudaError_t launch_knn_t(const void *base, const float *norms, int64_t n, const void *queries, int64_t nq,
-                         int64_t self0, int k, int32_t *ids, float *dists, int *err, cudaStream_t stream) {
+                         int64_t self0, int k, int32_t *ids, float *dists, const int *only, int *err,
+                         cudaStream_t stream) {
     const size_t smem = knn_smem_bytes(KS * 16);
-    cudaError_t e = cudaFuncSetAttribute(knn_bf16_kernel<KS, L2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = ensure_dyn_smem(reinterpret_cast<const void *>(knn_bf16_kernel<KS, L2>), (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = (nq + KBM - 1) / KBM;
     knn_bf16_kernel<KS, L2><<<(unsigned)grid, KNT, smem, stream>>>(
         reinterpret_cast<const __nv_bfloat16 *>(base), norms, n, reinterpret_cast<const __nv_bfloat16 *>(queries),
-        nq, self0, k, ids, dists, err);
+        nq, self0, k, ids, dists, only, err);
     return cudaGetLastError();
 }
 
@@ -454,21 +403,16 @@ cudaError_t launch_knn_t(const void *base, const float *norms, int64_t n, const 
 
 int64_t knn_norms_rows(int64_t n) { return (n + KBN - 1) / KBN * KBN; }
 
-cudaError_t launch_knn_bf16(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,
-                            int metric, int k, int32_t *ids, float *dists, float *norms, int *err,
-                            cudaStream_t stream) {
+cudaError_t launch_knn_scan(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,
+                            int metric, int k, int32_t *ids, float *dists, const float *norms, const int *only,
+                            int *err, cudaStream_t stream) {
     const bool l2 = metric == ANN_METRIC_L2;
-    if (l2) {
-        const int64_t np = knn_norms_rows(n);
-        bf16_row_norms<<<(unsigned)((np + 255) / 256), 256, 0, stream>>>(
-            reinterpret_cast<const __nv_bfloat16 *>(base), n, np, d, norms);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
 #define ANN_KNN_CASE(KS)                                                                                   \
     case KS:                                                                                               \
-        return l2 ? launch_knn_t<KS, true>(base, norms, n, queries, nq, self0, k, ids, dists, err, stream) \
-                  : launch_knn_t<KS, false>(base, norms, n, queries, nq, self0, k, ids, dists, err, stream);
+        return l2 ? launch_knn_t<KS, true>(base, norms, n, queries, nq, self0, k, ids, dists, only, err,   \
+                                           stream)                                                         \
+                  : launch_knn_t<KS, false>(base, norms, n, queries, nq, self0, k, ids, dists, only, err,  \
+                                            stream);
     switch (d / 16) {
         ANN_KNN_CASE(2)
         ANN_KNN_CASE(4)

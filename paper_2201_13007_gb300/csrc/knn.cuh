@@ -1,0 +1,29 @@
+// knn.cuh -- the brute-force k-NN over BF16 rows, for the host side.
+#pragma once
+
+#include "ann_internal.cuh"
+
+namespace ann {
+
+// knn_filter.cu: brute-force k-NN over BF16 rows (graph construction). A plan
+// gives the workspace a call needs (one device allocation, offsets of its
+// parts) and how the base and the queries are cut.
+struct KnnPlan {
+    int levels;        // the base is taken in levels + 1 nested samples
+    int chunk_blocks;  // blocks of 128 query rows per pass over the base
+    int splits;        // CTAs that share a block's tiles
+    size_t err, norms, bias, over, qnorm, margin, thr, kept_n, counts, kept, lists, bytes;
+};
+KnnPlan knn_plan(int64_t n, int64_t nq, int sms);
+// The int at ws + plan.err is set if a wait (2) or a merge (1) ran out.
+cudaError_t launch_knn_bf16(const KnnPlan &plan, void *ws, const void *base, int64_t n, int d, const void *queries,
+                            int64_t nq, int64_t self0, int metric, int k, int32_t *ids, float *dists, int sms,
+                            cudaStream_t stream);
+// knn.cu: the scan kernel, for the blocks of 128 query rows with only[block]
+// set. norms holds the base rows' squared norms (zeros up to
+// knn_norms_rows(n)); err is set to 1 if a CTA's merge rounds ran out.
+cudaError_t launch_knn_scan(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,
+                            int metric, int k, int32_t *ids, float *dists, const float *norms, const int *only,
+                            int *err, cudaStream_t stream);
+
+}  // namespace ann
