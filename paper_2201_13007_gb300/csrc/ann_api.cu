@@ -341,6 +341,8 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     if (p->l2_prefetch < 0 || p->l2_prefetch > 2)
         return fail(ANN_ERR_ARG, "l2_prefetch=%d not in {0, 1, 2}", p->l2_prefetch);
     a.l2_prefetch = p->l2_prefetch != 2;
+    a.row_lines = ann::prefetch_lines(x.d_pad * ann::storage_bytes(x.storage));
+    a.row_lines32 = ann::prefetch_lines(x.d_pad32 * 4);
     // neighbour groups serve the one-CTA sync kernel (the other kernels read every row by its id)
     a.hot_slot = (!async && csize == 1 && x.n_hot > 0) ? x.hot_slot : nullptr;
     a.group_prefetch = x.group_prefetch;

@@ -53,6 +53,9 @@ struct SmemLayout {
 
 __host__ __device__ inline int align16(int x) { return (x + 15) & ~15; }
 
+// The one-CTA sync kernel's control block, before the segments.
+static constexpr int kCtrlBytes = 256;
+
 // Shared memory of the one-CTA sync kernel with nw warps. The cand segment
 // holds each warp's fresh (id, row) pairs during a step (nw * ceil(Mcap * R /
 // nw) of them, one per 8-byte entry; the host makes Ccap at least that) and
@@ -70,7 +73,7 @@ __host__ __device__ inline SmemLayout sync_layout(int qfloats, int Lcap, int Cca
     s.dup_off = o;  o += align16(Ccap);
     s.hash_off = o; o += align16((1 << hash_bits) * slot_bytes);
     s.act_off = o;  o += align16(2 * Mcap * 4);
-    s.total = o;
+    s.total = kCtrlBytes + o;
     return s;
 }
 
@@ -102,6 +105,7 @@ struct SearchArgs {
     const int32_t *hot_slot; // neighbour groups: n entries, the group of a hot vertex or -1 (nullptr: none)
     int32_t group_prefetch;  // 0 = one bulk prefetch per hot vertex's block; 1 = the fresh rows only
     int32_t block_gather;    // one-CTA sync kernel: 1 = the CTA's fresh rows in one list gathered by all warps
+    int32_t row_lines, row_lines32;  // prefetch_lines of a stored row and of an FP32 row
     int32_t team_lanes;    // distance gather: log2 of the lanes that share one candidate row
     int32_t team_lanes32;  // the same for the FP32 rows of the re-rank
     int64_t *out_ids;
@@ -117,6 +121,16 @@ struct SearchArgs {
     int32_t qfloats;     // query buffer length
     SmemLayout sync_lay; // one-CTA sync kernel: segment offsets (kernel parameters, so no register holds them)
 };
+
+// 128-byte lines that a row can touch, where rows of row_bytes (a multiple of
+// 16) lie back to back from an aligned start; 0 for rows over 1 KB, which are
+// prefetched whole.
+inline int prefetch_lines(int row_bytes) {
+    if (row_bytes > 1024) return 0;
+    int g = 128;  // row starts are multiples of the largest power of two up to 128 that divides row_bytes
+    while (row_bytes % g) g >>= 1;
+    return (128 - g + row_bytes - 1) / 128 + 1;
+}
 
 inline int next_pow2(int x) {
     int p = 1;
@@ -180,13 +194,6 @@ cudaError_t launch_count_bad_adj(const int32_t *adj, int64_t count, int64_t n, u
                                  cudaStream_t stream);
 cudaError_t launch_count_in_degree(const int32_t *adj, int64_t count, int32_t *deg, cudaStream_t stream);
 
-// knn.cu: brute-force k-NN over BF16 rows (graph construction). norms holds
-// knn_norms_rows(n) floats for l2 (unused for inner product); err is a
-// device int set to 1 if a CTA's merge rounds ran out.
-int64_t knn_norms_rows(int64_t n);
-cudaError_t launch_knn_bf16(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,
-                            int metric, int k, int32_t *ids, float *dists, float *norms, int *err,
-                            cudaStream_t stream);
 cudaError_t launch_fill_groups(unsigned char *rows, float *scales, const int32_t *adj, const int32_t *hot,
                                int64_t n_hot, int32_t R, int64_t n, int32_t row_bytes, cudaStream_t stream);
 

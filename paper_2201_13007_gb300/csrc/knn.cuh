@@ -22,6 +22,7 @@ cudaError_t launch_knn_bf16(const KnnPlan &plan, void *ws, const void *base, int
 // knn.cu: the scan kernel, for the blocks of 128 query rows with only[block]
 // set. norms holds the base rows' squared norms (zeros up to
 // knn_norms_rows(n)); err is set to 1 if a CTA's merge rounds ran out.
+int64_t knn_norms_rows(int64_t n);
 cudaError_t launch_knn_scan(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,
                             int metric, int k, int32_t *ids, float *dists, const float *norms, const int *only,
                             int *err, cudaStream_t stream);

@@ -28,8 +28,7 @@ struct ClusterCtrl {
     int pub_n[2];      // survivors published in the step of this parity
     int pub_fresh[2];  // fresh vertices of this CTA in the step of this parity
     int pub_unsafe[2]; // this CTA's visited set may have forgotten a vertex (as of this step)
-    int unsafe, anydup, first_un, sel_last, wevals;
-    int wcnt[32];      // per-warp counts of the selection scan
+    int unsafe, anydup, repeats, first_un, sel_found, wevals;
     int rr_n;          // re-rank keys appended (rank 0, after the search; never read by another CTA)
     long long steps, expansions, dropped, t0;
     long long ph[4], tmark;  // rank 0's phase cycles (select, expand + distance, exchange, sort + merge)
@@ -63,7 +62,7 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = (int)keep_in_register(threadIdx.x), lane = tid & 31, warp = tid >> 5;
     const uint32_t row_bytes = (uint32_t)a.d_pad * ES;
     const uint32_t cpr = row_bytes / 16u;
     int off[10];
@@ -115,6 +114,7 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
         ctl.pub_fresh[0] = ctl.pub_fresh[1] = 0;
         ctl.unsafe = 0;
         ctl.first_un = 0;
+        ctl.repeats = 0;
         ctl.wevals = 0;
         ctl.ph[0] = ctl.ph[1] = ctl.ph[2] = ctl.ph[3] = 0;
     }
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     __syncthreads();
 
     int Mcur = a.M0 < Mmax ? a.M0 : Mmax;
-    int step = 0;
+    int step = 0, left = a.t;  // steps until M doubles
     int qlen = 1;
     const bool prof = a.phase_cycles != nullptr && rank == 0;
     if (prof && tid == 0) ctl.tmark = clock64();
@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     for (;;) {
         const int par = step & 1;
         // --- select (every CTA, identical): the first Mcur unchecked entries, all warps scanning
-        const int found = select_step<NW>(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, ctl.wcnt,
-                                               &ctl.sel_last);
+        const int found = select_step(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, &ctl.sel_found, tid);
         ANN_CPHASE(0)
         const int nact = found < Mcur ? found : Mcur;
         if (nact == 0) break;  // identical in every CTA: all leave the loop at the same step
@@ -161,11 +160,11 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
 
         // --- this CTA's own neighbours: adjacency -> visited set -> fresh lists -> distances -> published
         const int nf = expand_step<NW>(a, table, sel_id, nact, r_recip, row_bytes, fresh, nullptr, nullptr, C, rank,
-                                       &ctl.unsafe);
+                                       &ctl.unsafe, tid);
         if (lane == 0 && nf) atomicAdd(&ctl.wevals, nf);
         const entry_t limit = qlen >= L ? (Q[L - 1] & kMask) : kEmptyEntry;
         if (!gather_fixed<STORE, L2>(a.base, a.scales, cpr, a.team_lanes, qv, nullptr, fresh, nf, 0, 1, limit,
-                                     pub[par], &ctl.pub_n[par]))
+                                     pub[par], &ctl.pub_n[par], lane))
             warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, fresh, nf, a.team_lanes, limit, pub[par],
                                              &ctl.pub_n[par]);
         __syncthreads();
@@ -201,13 +200,13 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
             ctl.pub_n[par ^ 1] = 0;  // the next step's list (every CTA read it before this step's barrier)
             ctl.steps++;
             ctl.expansions += nact;
-            ctl.first_un = ctl.sel_last + 1;
+            ctl.first_un = sel_pos[nact - 1] + 1;
         }
         __syncthreads();
         ANN_CPHASE(2)
         if (tot > 0) {
-            const int ncl = sort_dedupe_merge<NT>(Q, qlen, uni, tot, cand, Qn, L, any_unsafe != 0, dup, &ctl.anydup,
-                                                  &ctl.dropped, &ctl.first_un);
+            const int ncl = sort_dedupe_merge<NT>(Q, qlen, uni, tot, cand, Qn, L, any_unsafe != 0, dup, &ctl.anydup, &ctl.repeats,
+                                                  &ctl.dropped, &ctl.first_un, tid);
             qlen = min(L, qlen + ncl);
             entry_t *t = Q;
             Q = Qn;
@@ -216,7 +215,10 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
             __syncthreads();
         }
         ANN_CPHASE(3)
-        if (step % a.t == 0) Mcur = min(2 * Mcur, Mmax);
+        if (--left == 0) {
+            Mcur = min(2 * Mcur, Mmax);
+            left = a.t;
+        }
     }
 #undef ANN_CPHASE
 
@@ -231,12 +233,12 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
             for (int i = tid; i < qlen; i += NT) {
                 const uint32_t id = entry_id(Q[i]);
                 cand[i] = (entry_t)id;
-                if (a.l2_prefetch) prefetch_row_l2(a.base32, (uint32_t)a.d_pad32 * 4u, id);
+                if (a.l2_prefetch) prefetch_row_l2(a.base32, (uint32_t)a.d_pad32 * 4u, id, a.row_lines32);
             }
             if (tid == 0) ctl.rr_n = 0;
             __syncthreads();
             if (!gather_fixed<ANN_STORE_F32, L2>(a.base32, nullptr, (uint32_t)a.d_pad32 / 4u, a.team_lanes32, qv,
-                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, uni, &ctl.rr_n))
+                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, uni, &ctl.rr_n, lane))
                 compute_keys_teams_m<ANN_STORE_F32, NT, L2, 2>(a.base32, nullptr, a.d_pad32, qv, cand, qlen,
                                                                a.team_lanes32, kEmptyEntry, uni, &ctl.rr_n);
             __syncthreads();

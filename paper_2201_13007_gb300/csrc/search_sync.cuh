@@ -8,8 +8,8 @@
 //
 // One step, inside one CTA of NW warps:
 //   select   warp 0 takes the first min(M_s, #unchecked) unchecked entries of
-//            the sorted queue by ballot + popc, starting past a prefix known to
-//            be checked;
+//            the sorted queue by ballot + popc, 128 entries a round, starting
+//            past a prefix known to be checked;
 //   expand   the step's M_s * R adjacency slots are split evenly over the
 //            warps (one lane per slot, coalesced int32 rows); each warp
 //            inserts its neighbours into the shared visited set and appends
@@ -20,10 +20,11 @@
 //            candidate below the queue's L-th entry to the CTA's survivor
 //            list. One barrier; then each warp marks its selected entries
 //            checked;
-//   sort     the survivors by (key, id): warp sort, run-rank sort or bitonic;
-//   merge    drop survivors whose id is already queued (only possible once
-//            the visited set forgot a vertex), then a merge-path merge of the
-//            queue and the survivors, truncated to L.
+//   merge    up to 128 survivors are ranked against the queue and each other
+//            and written to their places (merge_by_rank); more are sorted by
+//            warp runs and merged by merge path. Survivors whose id is already
+//            queued (only possible once the visited set forgot a vertex) are
+//            dropped, and the queue is cut to L.
 // The visited set may forget vertices (a direct-mapped cache evicts, an
 // open-addressing table is reset to the queued ids when half full); the queue
 // is then still the top-L of everything seen (a forgotten vertex that is met
@@ -41,25 +42,29 @@ struct Ctrl {
     int nfresh[2]; // block gather: fresh vertices appended in the step of this parity
     int hash_count;
     int do_reset;  // open addressing: the table is half full, reset it before the next select
-    int anydup;
+    int anydup, repeats;
     int unsafe;    // 1 once the visited set may have forgotten a vertex this query
     int first_un;  // every queue entry before this position is checked
     int qi, k, L, Mmax;  // the query and its settings (kept here, not in registers, across the step loop)
     int wevals;    // fresh vertices of this query, summed per warp and step
-    int sel_last;             // the step's selection: queue position of the last entry taken
-    int wcnt[32];             // per-warp counts of the selection scan
+    int sel_found;           // unchecked entries the step's selection saw
     // per-query counters, updated by thread 0 only
     long long steps, expansions, evals, resets, dropped, t0;
     long long ph[4], tmark;  // phase cycles (select, expand, distance, sort+merge) when requested
 };
 
+static_assert(sizeof(Ctrl) <= kCtrlBytes, "the control block lies before the segments of sync_layout");
+
 template <int NT, int STORE, bool L2>
 __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(const SearchArgs a) {
     constexpr int NW = NT / 32;
     constexpr uint32_t ES = STORE == ANN_STORE_F32 ? 4u : STORE == ANN_STORE_E4M3 ? 1u : 2u;
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ Ctrl ctl;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
+    unsigned char *const smem_ctl = static_cast<unsigned char *>(__cvta_shared_to_generic(
+        keep_in_register((uint32_t)__cvta_generic_to_shared(smem_dyn))));
+    Ctrl &ctl = *reinterpret_cast<Ctrl *>(smem_ctl);
+    unsigned char *const smem = smem_ctl + kCtrlBytes;
+    const int tid = (int)keep_in_register(threadIdx.x), lane = tid & 31, warp = tid >> 5;
     const uint32_t row_bytes = (uint32_t)a.d_pad * ES;
     const uint32_t cpr = row_bytes / 16u;
     const SmemLayout &lay = a.sync_lay;
@@ -97,6 +102,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
             ctl.evals = 1;
             ctl.unsafe = 0;
             ctl.first_un = 0;
+            ctl.repeats = 0;
             ctl.do_reset = 0;
             ctl.ph[0] = ctl.ph[1] = ctl.ph[2] = ctl.ph[3] = 0;
         }
@@ -106,6 +112,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
 
         const bool bad = ctl.k < 1 || ctl.k > a.k || ctl.L < ctl.k || ctl.L > a.L || ctl.Mmax < 1 || ctl.Mmax > a.M;
         if (bad) {
+#pragma unroll 1
             for (int i = tid; i < a.k; i += NT) {
                 a.out_ids[(size_t)qi * a.k + i] = -1;
                 a.out_dists[(size_t)qi * a.k + i] = __int_as_float(0x7f800000);
@@ -122,10 +129,12 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
 
         // query into shared memory, zero padded; clear the visited table
         const float *qg = a.queries + (size_t)qi * a.d;
+#pragma unroll 1
         for (int i = tid; i < a.qfloats; i += NT) qv[i] = i < a.d ? qg[i] : 0.f;
         {
             const int words = (H * a.slot_bytes) >> 2;
             const uint32_t empty = (a.slot_bytes < 4 || a.ways) ? 0u : kEmptySlot;
+#pragma unroll 1
             for (int i = tid; i < words; i += NT) table[i] = empty;
         }
         if (tid == 0) {
@@ -148,7 +157,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
         __syncthreads();
 
         int Mcur = a.M0 < ctl.Mmax ? a.M0 : ctl.Mmax;
-        int step = 0;
+        int step = 0, left = a.t;  // steps until M doubles
         int qlen = 1;  // the same in every thread
         entry_t *Q = Qa, *Qn = Qb;
         const bool prof = a.phase_cycles != nullptr;
@@ -164,8 +173,10 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
             // the direct-mapped cache never resets, it forgets by eviction
             // (decided by thread 0 after the last step's distance barrier, so every thread sees one value)
             if (ctl.do_reset) {
+#pragma unroll 1
                 for (int i = tid; i < H; i += NT) table[i] = kEmptySlot;
                 __syncthreads();
+#pragma unroll 1
                 for (int i = tid; i < qlen; i += NT) visited_insert(table, a.hash_bits, entry_id(Q[i]));
                 if (tid == 0) {
                     ctl.hash_count = qlen;
@@ -178,8 +189,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
             const int par = step & 1;
             // --- select: the first Mcur unchecked entries (rank order) of the stable queue, all warps
             // scanning from first_un (entries before it are all checked)
-            const int found = select_step<NW>(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, ctl.wcnt,
-                                                   &ctl.sel_last);
+            const int found = select_step(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, &ctl.sel_found, tid);
             const int nact = found < Mcur ? found : Mcur;
             if (nact == 0) break;  // no unchecked vertex left (identical in every warp)
             ANN_PHASE(0)
@@ -189,7 +199,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
             // list (+ L2 prefetch)
             const int nf = expand_step<NW>(a, table, sel_id, nact, r_recip, row_bytes, fresh,
                                            a.block_gather ? reinterpret_cast<uint2 *>(cand) : nullptr,
-                                           &ctl.nfresh[par], 1, 0, &ctl.unsafe);
+                                           &ctl.nfresh[par], 1, 0, &ctl.unsafe, tid);
             __syncwarp();
             if (lane == 0) {
                 if (nf) {
@@ -216,7 +226,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
                     gs = NW;
                 }
                 if (!gather_fixed<STORE, L2>(a.base, a.scales, cpr, a.team_lanes, qv, nullptr, gl, gn, gb, gs, limit,
-                                             surv, &ctl.ns[par]))
+                                             surv, &ctl.ns[par], lane))
                     warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, gl, gn, a.team_lanes, limit, surv,
                                                      &ctl.ns[par], gb, gs);
             }
@@ -229,14 +239,14 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
                 ctl.nfresh[par ^ 1] = 0;
                 ctl.steps++;
                 ctl.expansions += nact;
-                ctl.first_un = ctl.sel_last + 1;
+                ctl.first_un = sel_pos[nact - 1] + 1;
                 ctl.do_reset = a.visited_mode == 0 && ctl.hash_count * 2 > H;
             }
             if (ns > 0) {
                 // --- sort the survivors, drop ids already queued (only after the visited set forgot a vertex),
                 // merge into the other queue buffer truncated to L
                 const int ncl = sort_dedupe_merge<NT>(Q, qlen, surv, ns, cand, Qn, ctl.L, ctl.unsafe != 0, dup,
-                                                      &ctl.anydup, &ctl.dropped, &ctl.first_un);
+                                                      &ctl.anydup, &ctl.repeats, &ctl.dropped, &ctl.first_un, tid);
                 qlen = min(ctl.L, qlen + ncl);
                 entry_t *tmp = Q;
                 Q = Qn;
@@ -245,7 +255,10 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
                 __syncthreads();  // the marks and first_un are visible before the next select
             }
             ANN_PHASE(3)
-            if (step % a.t == 0) Mcur = min(2 * Mcur, ctl.Mmax);
+            if (--left == 0) {
+                Mcur = min(2 * Mcur, ctl.Mmax);
+                left = a.t;
+            }
         }
 #undef ANN_PHASE
 
@@ -253,16 +266,17 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
         const int k = ctl.k;
         const entry_t *res = Q;
         if (a.rerank) {
+#pragma unroll 1
             for (int i = tid; i < qlen; i += NT) {
                 const uint32_t id = entry_id(Q[i]);
                 cand[i] = (entry_t)id;
-                if (a.l2_prefetch) prefetch_row_l2(a.base32, (uint32_t)a.d_pad32 * 4u, id);
+                if (a.l2_prefetch) prefetch_row_l2(a.base32, (uint32_t)a.d_pad32 * 4u, id, a.row_lines32);
             }
             if (tid == 0) ctl.ns[0] = 0;
             __syncthreads();
             // every key is kept (limit = the empty entry), in whatever order the teams finish
             if (!gather_fixed<ANN_STORE_F32, L2>(a.base32, nullptr, (uint32_t)a.d_pad32 / 4u, a.team_lanes32, qv,
-                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, surv, &ctl.ns[0]))
+                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, surv, &ctl.ns[0], lane))
                 compute_keys_teams_m<ANN_STORE_F32, NT, L2, 2>(a.base32, nullptr, a.d_pad32, qv, cand, qlen,
                                                                a.team_lanes32, kEmptyEntry, surv, &ctl.ns[0]);
             __syncthreads();
@@ -280,6 +294,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
         }
         int64_t *oid = a.out_ids + (size_t)qi * a.k;
         float *odist = a.out_dists + (size_t)qi * a.k;
+#pragma unroll 1
         for (int i = tid; i < a.k; i += NT) {
             if (i < k && i < qlen) {
                 oid[i] = (int64_t)entry_id(res[i]);
