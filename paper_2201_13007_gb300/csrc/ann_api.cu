@@ -213,20 +213,22 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     if (p->merge_rule == 1 && !(p->patience >= 0.f))
         return fail(ANN_ERR_ARG, "patience must be >= 0 (or INFINITY) with merge_rule 1");
     if (async && M > 32) return fail(ANN_ERR_ARG, "async mode runs one warp per walker: M=%d > 32", M);
-    // cluster = 0 and at most 8 queries: each query on a cluster of 8 CTAs (4, 2 if fewer SMs), which the
-    // one-query latency measurements favour at every (L, M), when the cluster kernel runs the search as asked
-    // (sync, not persistent, no phase counters, no neighbour groups, a set-associative visited set); the
-    // results are those of one CTA per query. If that plan does not fit, one CTA per query.
-    if (p->cluster == 0 && nq >= 1 && nq <= 8 && !async && !p->persistent && !p->phase_cycles &&
+    // cluster = 0: while the SMs allow it each query runs on a cluster of CTAs, when the cluster kernel runs the search
+    // as asked (sync, not persistent, no phase counters, no neighbour groups, a set-associative visited set); the
+    // results are those of one CTA per query. If that plan does not fit, one CTA per query. The lines: a cluster of 8
+    // needs 8 free SMs of one GPC, and from 16 queries on they no longer all run at once (100 x 8 searches of 96-d
+    // BF16 rows, us, clusters of 8 / 4 / 2 / one CTA: 9 queries 114 / 115 / 120 / 132, 16: 195 / 116 / 122 / 134, 32:
+    // - / 133 / 141 / 151, 64: - / 232 / 144 / 155, 128: - / - / 257 / 164).
+    if (p->cluster == 0 && nq >= 1 && !async && !p->persistent && !p->phase_cycles &&
         (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0) {
-        for (int c = 8; c >= 2; c >>= 1) {
-            if ((int64_t)nq * c > sm_count()) continue;
+        const int sms = sm_count();
+        const int c = 12 * nq <= sms || (nq <= 8 && 8 * nq <= sms) ? 8 : 9 * nq <= 2 * sms ? 4 : 2 * nq <= sms ? 2 : 1;
+        if (c > 1) {
             ann_search_params pc = *p;
             pc.cluster = c;
             const std::string saved = g_err;
             if (plan_search(index, queries, nq, k, L, M, out_ids, out_dists, &pc, plan) == ANN_OK) return ANN_OK;
             g_err = saved;
-            break;
         }
     }
     const int csize = p->cluster > 1 ? p->cluster : 1;
@@ -234,13 +236,20 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
         return fail(ANN_ERR_ARG, "cluster=%d not in {0, 1, 2, 4, 8}", p->cluster);
     if (csize > 1 && async) return fail(ANN_ERR_ARG, "clusters are for sync mode only");
     int threads = p->threads;
-    // Automatic launch shape, from (threads, visited bits) sweeps on the 1M x 128 (10,000 queries)
-    // and 1M x 960 (1,000 queries) workloads. With at least 32 queries per SM the one-CTA sync
-    // kernel is fastest with small CTAs (more queries in flight per SM) and a 2^12-slot visited
-    // cache at every (L, M). With fewer queries each query's own latency counts: long queues or
-    // heavy steps (M * R rows of at least 256 KB) take 512 threads and 2^14 slots.
-    const bool many = !async && csize == 1 && nq >= 32LL * sm_count();
-    const bool heavy = L >= 384 || (int64_t)M * x.R * x.d_pad * ann::storage_bytes(x.storage) >= (256 << 10);
+    // Automatic launch shape of the one-CTA sync kernel, from sweeps of threads and visited bits over 152 to 10,000
+    // queries (1M x 96 BF16 and 128 FP32 rows, 200,000 x 960 FP16 and FP8 rows). An SM holds 1,024 threads of it, so
+    // with up to two queries per SM each takes 512 threads (256 if its steps have fewer than 256 slots), with up to
+    // four 256, and a visited set that lets them all reside. Beyond that throughput counts: 256 threads for steps of
+    // 1,024 slots or more, 512 where such steps would gather 768 KB of rows over 1 KB, else 128 or 256, whichever
+    // needs less time for its rounds of resident queries (a round of 128-thread CTAs takes 1.3 times one of 256).
+    // Against the former line at 32 queries per SM (us): 256 queries, L = 192, M = 16 290 -> 190; 456, L = 576, M = 32
+    // 508 -> 393; 2,432, L = 1024, M = 4 12,254 -> 5,771; 1,000 x 960-d FP8, L = 128, M = 8 1,107 -> 851.
+    const bool one = !async && csize == 1;
+    const int64_t sms = sm_count(), slots = (int64_t)M * x.R;
+    const int64_t row_bytes = (int64_t)x.d_pad * ann::storage_bytes(x.storage);
+    const bool few = nq <= 2 * sms;
+    const bool long_rows = row_bytes > 1024 && slots * row_bytes >= (768 << 10);
+    const bool heavy = L >= 384 || slots * row_bytes >= (256 << 10);  // long queues or heavy steps
     if (async) {
         // one warp per walker: T = M walkers, at least two warps
         int walkers = 2;
@@ -250,7 +259,24 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
             return fail(ANN_ERR_ARG, "threads=%d not in {64,...,1024}", threads);
         if (threads / 32 < M) return fail(ANN_ERR_ARG, "async mode needs threads >= 32*M");
     } else {
-        if (threads == 0) threads = many ? (M * x.R >= 1024 ? 256 : 128) : (heavy ? 512 : (M * x.R >= 1024 ? 256 : 128));
+        if (threads == 0 && !one) threads = heavy ? 512 : (slots >= 256 ? 256 : 128);
+        if (threads == 0) {
+            if (few) {
+                threads = slots >= 256 ? 512 : 256;
+            } else if (long_rows) {
+                threads = 512;
+            } else if (nq <= 4 * sms || slots >= 1024) {
+                threads = 256;
+            } else {
+                // queries resident per SM: 1,024 threads' worth, or what shared memory holds (queues, candidate
+                // lists, 16 KB of visited set, the query)
+                const int64_t smem = 16 * (int64_t)L + 17 * ann::next_pow2((int)slots) + (16 << 10) + x.d_pad32 * 4 +
+                                     1536;
+                const int64_t fit = std::max<int64_t>(1, (228 << 10) / smem);
+                const int64_t r128 = std::min<int64_t>(8, fit) * sms, r256 = std::min<int64_t>(4, fit) * sms;
+                threads = 13 * ((nq + r128 - 1) / r128) <= 10 * ((nq + r256 - 1) / r256) ? 128 : 256;
+            }
+        }
         if (threads != 64 && threads != 128 && threads != 256 && threads != 512)
             return fail(ANN_ERR_ARG, "threads=%d not in {64,128,256,512}", threads);
         if (csize > 1 && threads == 64) threads = 128;
@@ -289,7 +315,8 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     };
     int hb = p->hash_bits;
     if (hb == 0) {
-        if (many) {  // the most slots that fit in 16 KB (2^12 full ids or set words; 2^14 one-byte tags)
+        const bool packed = vmode >= 3 ? one && !few && !long_rows : one && nq >= 32 * sms;
+        if (packed) {  // the most slots that fit in 16 KB (2^12 full ids or set words; 2^14 one-byte tags)
             hb = 12;
             for (int b = 14; b > 12; --b)
                 if ((1 << b) * slot_bytes_for(b) <= (16 << 10)) {
@@ -297,11 +324,11 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
                     break;
                 }
             while (vmode == 4 && ways_for(hb) < 2) ++hb;  // more sets leave more bits per tag
-        } else if (vmode == 4) {  // 2^13 sets hold 24,576 tags in 32 KB; 2^14 for long queues or heavy steps
-            hb = heavy ? 14 : 13;
+        } else if (vmode == 4) {  // 2^13 sets hold 24,576 tags in 32 KB; 2^14 for clusters' long queues or heavy steps
+            hb = !one && heavy ? 14 : 13;
             while (ways_for(hb) < 2) ++hb;
         } else {
-            hb = heavy ? 14 : (M * x.R >= 1024 ? 13 : 12);
+            hb = heavy ? 14 : (slots >= 1024 ? 13 : 12);
         }
     }
     if (hb < 8 || hb > 15) return fail(ANN_ERR_ARG, "hash_bits=%d outside [8, 15]", hb);
