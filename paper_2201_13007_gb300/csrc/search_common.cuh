@@ -465,31 +465,15 @@ __device__ void block_bitonic_sort(entry_t *s, int P) {
 // Number of entries of sorted A[0..n) that are below x, comparing with the
 // checked flag masked off.
 __device__ __forceinline__ int count_below(const entry_t *A, int n, entry_t x) {
-    int lo = 0, hi = n;
+    int lo = 0;
 #pragma unroll 1
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if ((A[mid] & kMask) < x) lo = mid + 1;
-        else hi = mid;
+    for (int hi = n; lo < hi;) {
+        const int mid = (lo + hi) >> 1;
+        const bool below = (A[mid] & kMask) < x;
+        lo = below ? mid + 1 : lo;
+        hi = below ? hi : mid;
     }
     return lo;
-}
-
-// The same count with three probes in flight at a time: half of the round
-// trips to shared memory of the binary search, for code whose time they are.
-__device__ __forceinline__ int count_below4(const entry_t *A, int n, entry_t x) {
-    int s = 1;
-    while (4 * s <= n) s *= 4;
-    int p = 0;
-#pragma unroll 1
-    for (; s > 0; s >>= 2) {
-        const int i = p + s - 1;
-        const bool b0 = i < n && (A[i] & kMask) < x;
-        const bool b1 = i + s < n && (A[i + s] & kMask) < x;
-        const bool b2 = i + 2 * s < n && (A[i + 2 * s] & kMask) < x;
-        p += s * (b0 + b1 + b2);
-    }
-    return p;
 }
 
 __device__ __forceinline__ int64_t global_ns() {
@@ -903,7 +887,7 @@ __device__ __forceinline__ void warp_keys_fixed(const void *rows, const float *s
 #pragma unroll
             for (int off = TS >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(kFull, r, off);
             e[u] = pack_entry(L2 ? r : -r, id[u]);
-            keep[u] = tl == 0 && c0 + u * c_step + team < nf && e[u] < limit;
+            keep[u] = (tl == 0) & (c0 + u * c_step + team < nf) & (e[u] < limit);
             bal[u] = __ballot_sync(kFull, keep[u]);
             n += __popc(bal[u]);
         }
@@ -1006,7 +990,7 @@ __device__ __forceinline__ int select_step(const entry_t *Q, int qlen, int first
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int r = found + __popc(bal[c] & ((1u << lane) - 1u));
-                if ((int)e[c] >= 0 && r < Mcur) {
+                if (((int)e[c] >= 0) & (r < Mcur)) {
                     sel_id[r] = (int)e[c];
                     sel_pos[r] = b + c * 32 + lane;
                 }
@@ -1019,45 +1003,68 @@ __device__ __forceinline__ int select_step(const entry_t *Q, int qlen, int first
     return *sel_found;
 }
 
+// Shared-memory atomics and an L2 prefetch under a predicate instead of a
+// branch, so that several are in flight (`old` is kept where p is false).
+__device__ __forceinline__ void cas_if(bool p, uint32_t &old, uint32_t addr, uint32_t cmp, uint32_t val) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %4, 0;\n@p atom.shared.cas.b32 %0, [%1], %2, %3;\n}\n"
+                 : "+r"(old)
+                 : "r"(addr), "r"(cmp), "r"(val), "r"((int)p)
+                 : "memory");
+}
+__device__ __forceinline__ void exch_if(bool p, uint32_t &old, uint32_t addr, uint32_t val) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %3, 0;\n@p atom.shared.exch.b32 %0, [%1], %2;\n}\n"
+                 : "+r"(old)
+                 : "r"(addr), "r"(val), "r"((int)p)
+                 : "memory");
+}
+__device__ __forceinline__ void prefetch_if(bool p, size_t addr) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.s32 p, %1, 0;\n@p prefetch.global.L2 [%0];\n}\n" ::"l"(addr), "r"((int)p));
+}
+
 // The inserts of KA vertices of a lane (negative: none); bit kk of the result
 // is set if the visited set did not hold u[kk], and forgot if another vertex
 // may have fallen out. The two forms that searches use by default are inserted
-// with all of the lane's words in flight: one after another, their round trips
-// to shared memory were most of an expansion.
+// with all of the lane's words in flight and without branches around them: one
+// after another, their round trips to shared memory were most of an expansion.
 template <int KA>
 __device__ __forceinline__ unsigned visit_batch(uint32_t *table, const SearchArgs &a, const int (&u)[KA],
                                                 bool &forgot) {
     unsigned fr = 0;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(table);
     if (a.ways) {  // set-associative words of 2 or 3 tags, see visited_assoc
         const int b = a.hash_bits + a.tag_bits, fw = a.tag_bits + 1, top = (a.ways - 1) * fw;
         const uint32_t hmask = b < 32 ? (1u << b) - 1u : 0xFFFFFFFFu;
         const uint32_t fmask = (1u << fw) - 1u;
         const uint32_t wmask = a.ways * fw >= 32 ? 0xFFFFFFFFu : (1u << (a.ways * fw)) - 1u;
-        uint32_t old[KA], set[KA], tag[KA];
+        // a one in each field: the tag times it is the tag in every field, and a word that differs from that in every
+        // field has no zero field: (x - ones) & ~x has no field's top bit
+        const uint32_t ones = 1u | 1u << fw | 1u << top, highs = ones << (fw - 1);
+        uint32_t old[KA], h[KA], prev[KA];
 #pragma unroll
         for (int kk = 0; kk < KA; ++kk) {
-            const uint32_t h = ((uint32_t)u[kk] * 0x9E3779B1u) & hmask;
-            set[kk] = h >> a.tag_bits;
-            tag[kk] = (h & (fmask >> 1)) + 1u;
-            old[kk] = u[kk] >= 0 ? *reinterpret_cast<volatile uint32_t *>(table + set[kk]) : 0u;
-        }
-        uint32_t prev[KA];
-#pragma unroll
-        for (int kk = 0; kk < KA; ++kk) {
-            // the top field of a two-tag word is its second: compared twice
-            const bool seen = (old[kk] & fmask) == tag[kk] || ((old[kk] >> fw) & fmask) == tag[kk] ||
-                              ((old[kk] >> top) & fmask) == tag[kk];
-            if (u[kk] >= 0 && !seen) {
-                fr |= 1u << kk;
-                prev[kk] = atomicCAS(table + set[kk], old[kk], ((old[kk] << fw) | tag[kk]) & wmask);
-            }
+            h[kk] = ((uint32_t)u[kk] * 0x9E3779B1u) & hmask;  // any u gives a word of the table
+            old[kk] = *reinterpret_cast<volatile uint32_t *>(table + (h[kk] >> a.tag_bits));
         }
 #pragma unroll
         for (int kk = 0; kk < KA; ++kk) {
-            if (!(fr >> kk & 1u)) continue;
-            if (prev[kk] == old[kk]) {
-                forgot |= ((old[kk] >> top) & fmask) != 0u;
-            } else {  // another insert changed the word in between
+            const uint32_t tag = (h[kk] & (fmask >> 1)) + 1u;
+            const uint32_t x = old[kk] ^ (tag * ones);
+            const bool add = (u[kk] >= 0) & (((x - ones) & ~x & highs) == 0u);
+            fr |= (unsigned)add << kk;
+            prev[kk] = old[kk];
+            cas_if(add, prev[kk], base + (h[kk] >> a.tag_bits) * 4u, old[kk], ((old[kk] << fw) | tag) & wmask);
+        }
+        unsigned again = 0;
+#pragma unroll
+        for (int kk = 0; kk < KA; ++kk) {
+            const bool add = fr >> kk & 1u;
+            again |= (unsigned)(prev[kk] != old[kk]) << kk;  // another insert changed the word in between
+            forgot |= add & (((old[kk] >> top) & fmask) != 0u);
+        }
+        if (again) {
+#pragma unroll
+            for (int kk = 0; kk < KA; ++kk) {
+                if (!(again >> kk & 1u)) continue;
                 const int ins = visit_set(table, a, (uint32_t)u[kk]);
                 if (ins == 0) fr &= ~(1u << kk);
                 forgot |= ins >= 2;
@@ -1068,15 +1075,17 @@ __device__ __forceinline__ unsigned visit_batch(uint32_t *table, const SearchArg
     if (a.visited_mode != 0 && a.slot_bytes == 4) {  // direct-mapped ids, see visited_exchange
         uint32_t old[KA];
 #pragma unroll
-        for (int kk = 0; kk < KA; ++kk)
-            if (u[kk] >= 0)
-                old[kk] = atomicExch(table + (((uint32_t)u[kk] * 0x9E3779B1u) >> (32 - a.hash_bits)), (uint32_t)u[kk]);
+        for (int kk = 0; kk < KA; ++kk) {
+            old[kk] = (uint32_t)u[kk];
+            exch_if(u[kk] >= 0, old[kk], base + (((uint32_t)u[kk] * 0x9E3779B1u) >> (32 - a.hash_bits)) * 4u,
+                    (uint32_t)u[kk]);
+        }
 #pragma unroll
-        for (int kk = 0; kk < KA; ++kk)
-            if (u[kk] >= 0 && old[kk] != (uint32_t)u[kk]) {
-                fr |= 1u << kk;
-                forgot |= old[kk] != kEmptySlot;
-            }
+        for (int kk = 0; kk < KA; ++kk) {
+            const bool add = old[kk] != (uint32_t)u[kk];
+            fr |= (unsigned)add << kk;
+            forgot |= add & (old[kk] != kEmptySlot);
+        }
         return fr;
     }
 #pragma unroll
@@ -1117,30 +1126,33 @@ __device__ __forceinline__ int expand_step(const SearchArgs &a, uint32_t *table,
         int u[KA];
         uint32_t urow[KA];  // the row holding u's vector: u, or its copy in a neighbour group
 #pragma unroll
+        for (int kk = 0; kk < KA; ++kk) {  // all loads first; a lane past the end repeats the last slot
+            const uint32_t i = (uint32_t)min(b0 + kk * 32 + lane, end - 1);
+            const uint32_t j = __umulhi(i, r_recip);
+            u[kk] = __ldg(a.adj + (size_t)(uint32_t)sel_id[j] * (uint32_t)R + (i - j * (uint32_t)R));
+        }
+#pragma unroll
         for (int kk = 0; kk < KA; ++kk) {
-            const int i = b0 + kk * 32 + lane;
-            u[kk] = -1;
-            urow[kk] = 0;
-            if (i < end) {
+            const bool other = (owners > 1) & (((uint32_t)u[kk] & (uint32_t)(owners - 1)) != (uint32_t)owner);
+            if ((b0 + kk * 32 + lane >= end) | other) u[kk] = -1;
+            urow[kk] = (uint32_t)u[kk];
+        }
+        if (a.hot_slot) {
+            // a hot vertex: its neighbours' rows lie in one block after the base rows, in adjacency order; one bulk
+            // prefetch (from the lane with its first slot) asks L2 for the block
+#pragma unroll
+            for (int kk = 0; kk < KA; ++kk) {
+                const int i = b0 + kk * 32 + lane;
+                if (i >= end) continue;
                 const uint32_t j = __umulhi((uint32_t)i, r_recip);
                 const uint32_t slot = (uint32_t)i - j * (uint32_t)R;
-                const uint32_t v = (uint32_t)sel_id[j];
-                u[kk] = __ldg(a.adj + (size_t)v * (uint32_t)R + slot);
-                if (owners > 1 && u[kk] >= 0 && ((uint32_t)u[kk] & (uint32_t)(owners - 1)) != (uint32_t)owner)
-                    u[kk] = -1;
-                urow[kk] = (uint32_t)u[kk];
-                if (a.hot_slot) {
-                    // a hot vertex: its neighbours' rows lie in one block after the base rows, in adjacency
-                    // order; one bulk prefetch (from the lane with its first slot) asks L2 for the block
-                    const int hs = __ldg(a.hot_slot + v);
-                    if (hs >= 0) {
-                        const uint32_t r0 = (uint32_t)a.n + (uint32_t)hs * (uint32_t)R;
-                        urow[kk] = r0 + slot;
-                        if (slot == 0 && a.l2_prefetch && a.group_prefetch == 0)
-                            prefetch_range_l2(static_cast<const char *>(a.base) + (size_t)r0 * row_bytes,
-                                              (uint32_t)R * row_bytes);
-                    }
-                }
+                const int hs = __ldg(a.hot_slot + (uint32_t)sel_id[j]);
+                if (hs < 0) continue;
+                const uint32_t r0 = (uint32_t)a.n + (uint32_t)hs * (uint32_t)R;
+                urow[kk] = r0 + slot;
+                if (slot == 0 && a.l2_prefetch && a.group_prefetch == 0)
+                    prefetch_range_l2(static_cast<const char *>(a.base) + (size_t)r0 * row_bytes,
+                                      (uint32_t)R * row_bytes);
             }
         }
         bool forgot = false;
@@ -1161,12 +1173,43 @@ __device__ __forceinline__ int expand_step(const SearchArgs &a, uint32_t *table,
         uint2 *dst = block ? block : fresh;
 #pragma unroll
         for (int kk = 0; kk < KA; ++kk) {
-            if (fr >> kk & 1u) {
-                dst[pos + __popc(bal[kk] & ((1u << lane) - 1u))] = make_uint2((uint32_t)u[kk], urow[kk]);
-                if (a.l2_prefetch && (urow[kk] < (uint32_t)a.n || a.group_prefetch))
-                    prefetch_row_l2(a.base, row_bytes, urow[kk], a.row_lines);
-            }
+            if (fr >> kk & 1u) dst[pos + __popc(bal[kk] & ((1u << lane) - 1u))] = make_uint2((uint32_t)u[kk], urow[kk]);
             pos += __popc(bal[kk]);
+        }
+        if (a.l2_prefetch) {
+            unsigned ask = fr;  // rows to ask for one by one: not those of a group that was asked for whole
+            if (a.hot_slot && !a.group_prefetch) {
+#pragma unroll
+                for (int kk = 0; kk < KA; ++kk)
+                    if (urow[kk] >= (uint32_t)a.n) ask &= ~(1u << kk);
+            }
+            if (a.row_lines) {
+                const size_t rows = __cvta_generic_to_global(a.base);
+                if (a.row_lines <= 2) {  // the last byte stands for the last line, see prefetch_row_l2
+                    const uint32_t last = row_bytes - 1u;
+#pragma unroll
+                    for (int kk = 0; kk < KA; ++kk)
+                        prefetch_if((ask >> kk & 1u) & (a.row_lines == 2), rows + (size_t)urow[kk] * row_bytes);
+#pragma unroll
+                    for (int kk = 0; kk < KA; ++kk)
+                        prefetch_if(ask >> kk & 1u, rows + (size_t)urow[kk] * row_bytes + last);
+                } else {
+                    // row by row: 10,000 queries over 512-byte rows take 9.51 ms this way and 9.95 line by line (rows of
+                    // two lines, 256 bytes: 5.75 and 5.70)
+#pragma unroll
+                    for (int kk = 0; kk < KA; ++kk) {
+                        const size_t row = rows + (size_t)urow[kk] * row_bytes;
+#pragma unroll 1
+                        for (int l = 1; l < a.row_lines; ++l)
+                            prefetch_if(ask >> kk & 1u, row + (uint32_t)(l - 1) * 128u);
+                        prefetch_if(ask >> kk & 1u, row + (row_bytes - 1u));
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int kk = 0; kk < KA; ++kk)
+                    if (ask >> kk & 1u) prefetch_row_l2(a.base, row_bytes, urow[kk], 0);
+            }
         }
         nf += wtot;
     }
@@ -1192,7 +1235,7 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
     int p = 0, kept = ns;
     if (tid < ns) {
         e = surv[tid];
-        p = count_below4(Q, qlen, e);
+        p = count_below(Q, qlen, e);
     }
     if (unsafe) {
         const bool drop = tid < ns && p < qlen && (Q[p] & kMask) == e;
@@ -1230,13 +1273,13 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
         const int per = (qlen + NT - 1) / NT, i1 = min((tid + 1) * per, qlen);
         int i = tid * per;
         if (i < i1) {
-            int lo = 0, s = 1;  // survivors placed at or before position i
-            while (4 * s <= kept) s *= 4;
+            int lo = 0;  // survivors placed at or before position i
 #pragma unroll 1
-            for (; s > 0; s >>= 2) {
-                const int j = lo + s - 1;
-                lo += s * ((j < kept && (where[j] & 0xFFFF) <= i) + (j + s < kept && (where[j + s] & 0xFFFF) <= i) +
-                           (j + 2 * s < kept && (where[j + 2 * s] & 0xFFFF) <= i));
+            for (int hi = kept; lo < hi;) {
+                const int mid = (lo + hi) >> 1;
+                const bool below = (where[mid] & 0xFFFF) <= i;
+                lo = below ? mid + 1 : lo;
+                hi = below ? hi : mid;
             }
 #pragma unroll 1
             for (; i < i1; ++i) {
@@ -1259,7 +1302,8 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
 }
 
 // The ns (> 0) survivors in surv, in no order, are merged into the sorted
-// queue Q[0..qlen): up to 128 by rank (merge_by_rank), more sorted first (one a
+// queue Q[0..qlen): up to 128 (256 in CTAs of 512 threads) by rank
+// (merge_by_rank), more sorted first (one a
 // thread: warp runs plus binary-search ranks into `scratch`; above that warp
 // runs merged pairwise between surv and `scratch`) and merged by merge path.
 // When `unsafe` (the visited set may have forgotten a vertex) survivors whose id
