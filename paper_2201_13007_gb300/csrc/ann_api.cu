@@ -259,7 +259,11 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
             return fail(ANN_ERR_ARG, "threads=%d not in {64,...,1024}", threads);
         if (threads / 32 < M) return fail(ANN_ERR_ARG, "async mode needs threads >= 32*M");
     } else {
-        if (threads == 0 && !one) threads = heavy ? 512 : (slots >= 256 ? 256 : 128);
+        // clusters: 512 threads for wide steps or heavy rows, 256 for steps of 256 slots or long queues, else 128 (clusters
+        // of 8, 512 / 256 / 128 threads, us: L = 576, M = 64 122 / 132 / -, L = 576, M = 32 156 / 157 / -, L = 192, M = 16
+        // 128 / 115 / -, L = 1024, M = 4 1104 / 1020 / 1072)
+        if (threads == 0 && !one)
+            threads = slots >= 2048 || slots * row_bytes >= (512 << 10) ? 512 : (slots >= 256 || L >= 384 ? 256 : 128);
         if (threads == 0) {
             if (few) {
                 threads = slots >= 256 ? 512 : 256;

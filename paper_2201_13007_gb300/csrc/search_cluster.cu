@@ -8,11 +8,10 @@
 // kernel, but vertex u belongs to CTA (u mod C): only its owner inserts it
 // into its visited set and gathers its row, so a step's row gathers are
 // spread over C SMs. Each CTA filters its new candidates by the current L-th
-// entry and publishes them in shared memory (double-buffered by step parity);
-// after one cluster barrier every CTA reads all published lists through
-// distributed shared memory, sorts their union, drops ids already queued
-// (when some owner's visited set forgot a vertex) and merges: the same inputs
-// in every CTA, so the queues stay identical and every CTA takes the same
+// entry and writes what is left into every CTA's shared memory (double-buffered
+// by step parity); after one cluster barrier every CTA has all lists, drops ids
+// already queued (when some owner's visited set forgot a vertex) and merges: the
+// same inputs in every CTA, so the queues stay identical and every CTA takes the same
 // number of steps and barriers. Because ownership partitions the vertices,
 // the union of the CTAs' new candidates is exactly the one-CTA kernel's, and
 // the results are identical to it.
@@ -25,18 +24,23 @@ namespace cg = cooperative_groups;
 namespace ann {
 
 struct ClusterCtrl {
-    int pub_n[2];      // survivors published in the step of this parity
-    int pub_fresh[2];  // fresh vertices of this CTA in the step of this parity
-    int pub_unsafe[2]; // this CTA's visited set may have forgotten a vertex (as of this step)
+    int pub_n;         // survivors of this CTA in this step
+    int cnt[2][8];     // per parity and CTA, written by that CTA: its survivors; kClusterUnsafe: its set may have forgotten
     int unsafe, anydup, repeats, first_un, sel_found, wevals;
     int rr_n;          // re-rank keys appended (rank 0, after the search; never read by another CTA)
-    long long steps, expansions, dropped, t0;
+    long long steps, expansions, dropped, own_dropped, t0;
     long long ph[4], tmark;  // rank 0's phase cycles (select, expand + distance, exchange, sort + merge)
 };
 
+static constexpr int kClusterUnsafe = 1 << 30;
+// Survivors of a step after which the next step's lists are sorted by their owners (numbers change little from step to
+// step): merging C sorted runs then takes no sort of the union. One query, L = 576, M = 64 on 8 CTAs of 512 threads: 130
+// us reading and sorting the union in every CTA, 126 with the lists written instead of read, 122 with sorted runs.
+static constexpr int kClusterRuns = 96;
+
 // Segments: query, two queue buffers, per-warp fresh lists (then sort
-// scratch), published survivors (two parities), the gathered union, dedupe
-// flags, the visited set (this CTA's vertices) and the selection.
+// scratch), this CTA's survivors (then the union in one piece), every CTA's
+// survivors as they wrote them (two parities), dedupe flags, the visited set (this CTA's vertices) and the selection.
 __host__ __device__ inline int cluster_smem_bytes(int qfloats, int Lcap, int Ccap, int hash_bits, int Mcap,
                                                   int *off) {
     int o = 0;
@@ -44,9 +48,9 @@ __host__ __device__ inline int cluster_smem_bytes(int qfloats, int Lcap, int Cca
     off[1] = o; o += align16(Lcap * 8);             // queue
     off[2] = o; o += align16(Lcap * 8);             // next queue
     off[3] = o; o += align16(Ccap * 8);             // fresh (id, row) pairs; sort scratch; re-rank ids
-    off[4] = o; o += align16(Ccap * 8);             // published survivors, parity 0
-    off[5] = o; o += align16(Ccap * 8);             // published survivors, parity 1
-    off[6] = o; o += align16(Ccap * 8);             // gathered union; re-rank keys
+    off[4] = o; o += align16(Ccap * 8);             // own survivors; the union; re-rank keys
+    off[5] = o; o += align16(Ccap * 8);             // every CTA's survivors, parity 0
+    off[6] = o; o += align16(Ccap * 8);             // every CTA's survivors, parity 1
     off[7] = o; o += align16(Ccap);                 // dup flags
     off[8] = o; o += align16((1 << hash_bits) * 4); // visited set (own vertices)
     off[9] = o; o += align16(2 * Mcap * 4);         // selected vertices and their queue positions
@@ -71,8 +75,10 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     entry_t *Q = reinterpret_cast<entry_t *>(smem + off[1]);
     entry_t *Qn = reinterpret_cast<entry_t *>(smem + off[2]);
     entry_t *cand = reinterpret_cast<entry_t *>(smem + off[3]);
-    entry_t *pub[2] = {reinterpret_cast<entry_t *>(smem + off[4]), reinterpret_cast<entry_t *>(smem + off[5])};
-    entry_t *uni = reinterpret_cast<entry_t *>(smem + off[6]);
+    entry_t *pub = reinterpret_cast<entry_t *>(smem + off[4]);
+    entry_t *uni[2] = {reinterpret_cast<entry_t *>(smem + off[5]), reinterpret_cast<entry_t *>(smem + off[6])};
+    const int seg = a.Ccap / C;  // entries of each CTA in uni[]
+    const int lc = C == 8 ? 3 : C == 4 ? 2 : 1;
     unsigned char *dup = smem + off[7];
     uint32_t *table = reinterpret_cast<uint32_t *>(smem + off[8]);
     int *sel_id = reinterpret_cast<int *>(smem + off[9]);
@@ -109,9 +115,8 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
 
     if (tid == 0) {
         ctl.t0 = global_ns();
-        ctl.steps = ctl.expansions = ctl.dropped = 0;
-        ctl.pub_n[0] = ctl.pub_n[1] = 0;
-        ctl.pub_fresh[0] = ctl.pub_fresh[1] = 0;
+        ctl.steps = ctl.expansions = ctl.dropped = ctl.own_dropped = 0;
+        ctl.pub_n = 0;
         ctl.unsafe = 0;
         ctl.first_un = 0;
         ctl.repeats = 0;
@@ -128,17 +133,18 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     __syncthreads();
     // the entry point: every CTA computes the same key; its owner marks it visited
     if (warp == 0)
-        warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, fresh, 1, a.team_lanes, kEmptyEntry, uni,
-                                         &ctl.pub_n[1]);
+        warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, fresh, 1, a.team_lanes, kEmptyEntry, pub,
+                                         &ctl.pub_n);
     __syncthreads();
     if (tid == 0) {
-        Q[0] = uni[0];
-        ctl.pub_n[1] = 0;
+        Q[0] = pub[0];
+        ctl.pub_n = 0;
         if ((int)(a.entry % C) == rank) visit_set(table, a, (uint32_t)a.entry);
     }
-    __syncthreads();
+    cluster.sync();  // no CTA writes into another before that one has begun
 
     int Mcur = a.M0 < Mmax ? a.M0 : Mmax;
+    int last_tot = 0;  // the union of the step before
     int step = 0, left = a.t;  // steps until M doubles
     int qlen = 1;
     const bool prof = a.phase_cycles != nullptr && rank == 0;
@@ -163,50 +169,120 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
                                        &ctl.unsafe, tid);
         if (lane == 0 && nf) atomicAdd(&ctl.wevals, nf);
         const entry_t limit = qlen >= L ? (Q[L - 1] & kMask) : kEmptyEntry;
-        if (!gather_fixed<STORE, L2>(a.base, a.scales, cpr, a.team_lanes, qv, nullptr, fresh, nf, 0, 1, limit,
-                                     pub[par], &ctl.pub_n[par], lane))
-            warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, fresh, nf, a.team_lanes, limit, pub[par],
-                                             &ctl.pub_n[par]);
+        if (!gather_fixed<STORE, L2>(a.base, a.scales, cpr, a.team_lanes, qv, nullptr, fresh, nf, 0, 1, limit, pub,
+                                     &ctl.pub_n, lane))
+            warp_keys_append_m<STORE, 4, L2>(a.base, a.scales, cpr, qv, fresh, nf, a.team_lanes, limit, pub,
+                                             &ctl.pub_n);
         __syncthreads();
-        if (tid == 0) ctl.pub_unsafe[par] = ctl.unsafe;
         ANN_CPHASE(1)
-        cluster.sync();  // every CTA's survivors of this step are published
-        // gather the union in rank order (the same order in every CTA): every thread reads all
-        // counts at once, then copies its share of all lists in one pass (two remote round trips)
-        int cn[8];
-        int tot = 0, any_unsafe = 0;
+        // --- exchange: each CTA writes its survivors into its segment of every CTA's uni[par] and its count beside them;
+        // after one cluster barrier all of it is local (reading the other CTAs' counts and lists after the barrier
+        // instead took two remote round trips more). After a step with many survivors the
+        // segments are sorted first (and rid of repeats), each by its own CTA.
+        int n = ctl.pub_n;
+        const bool unsafe = ctl.unsafe != 0, runs = last_tot > kClusterRuns;
+        const entry_t *mine = pub;
+        if (runs && (n > 1 || (unsafe && n > 0)))
+            mine = sort_dedupe<NT>(Q, qlen, pub, &n, cand, unsafe, dup, &ctl.anydup, &ctl.own_dropped, tid);
+        if (n <= seg)
+            for (int x = tid; x < n * C; x += NT)
+                cluster.map_shared_rank(uni[par], x & (C - 1))[rank * seg + (x >> lc)] = mine[x >> lc];
+        if (tid < C) cluster.map_shared_rank(ctl.cnt[par], tid)[rank] = n | (unsafe ? kClusterUnsafe : 0);
+        cluster.sync();
+        int cn[8], at[8];  // each CTA's survivors, and where they begin in uni[par]
+        int tot = 0, most = 0;
+        bool any_unsafe = false;
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            cn[r] = 0;
-            if (r < C) {
-                cn[r] = *cluster.map_shared_rank(&ctl.pub_n[par], r);
-                any_unsafe |= *cluster.map_shared_rank(&ctl.pub_unsafe[par], r);
+            const int c = r < C ? ctl.cnt[par][r] : 0;
+            any_unsafe |= (c & kClusterUnsafe) != 0;
+            cn[r] = c & ~kClusterUnsafe;
+            at[r] = r * seg;
+            tot += cn[r];
+            most = max(most, cn[r]);
+        }
+        if (most > seg) {  // one CTA has more than its share: all lists again, one behind the other
+            int o = 0, to = 0;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                at[r] = o;
+                if (r == rank) to = o;
+                o += cn[r];
             }
+            for (int x = tid; x < n * C; x += NT)
+                cluster.map_shared_rank(uni[par], x & (C - 1))[to + (x >> lc)] = mine[x >> lc];
+            cluster.sync();
         }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) tot += cn[r];
-        for (int i = tid; i < tot; i += NT) {
-            int r = 0, base_r = 0;
-#pragma unroll
-            for (int rr = 0; rr < 7; ++rr)
-                if (r == rr && i - base_r >= cn[rr]) {
-                    base_r += cn[rr];
-                    r = rr + 1;
-                }
-            uni[i] = cluster.map_shared_rank(pub[par], r)[i - base_r];
-        }
+        last_tot = tot;
         if (tid < nact) Q[sel_pos[tid]] |= kChecked;  // the selection is taken: mark it
         if (tid == 0) {
-            ctl.pub_n[par ^ 1] = 0;  // the next step's list (every CTA read it before this step's barrier)
+            ctl.pub_n = 0;
             ctl.steps++;
             ctl.expansions += nact;
             ctl.first_un = sel_pos[nact - 1] + 1;
         }
-        __syncthreads();
         ANN_CPHASE(2)
-        if (tot > 0) {
-            const int ncl = sort_dedupe_merge<NT>(Q, qlen, uni, tot, cand, Qn, L, any_unsafe != 0, dup, &ctl.anydup, &ctl.repeats,
-                                                  &ctl.dropped, &ctl.first_un, tid);
+        if (tot > 0 && runs) {
+            // --- merge of sorted runs: a survivor's rank is its place in its own run and the entries below it in the
+            // others (ownership partitions the vertices: no id is in two runs)
+            int *where = reinterpret_cast<int *>(cand);
+            int top = 1;
+            while (2 * top <= most) top *= 2;
+            for (int x = tid; x < tot; x += NT) {
+                int own = 0, i = x;
+#pragma unroll
+                for (int r = 0; r < 7; ++r)
+                    if (own == r && i >= cn[r]) {
+                        i -= cn[r];
+                        own = r + 1;
+                    }
+                int from = 0;
+#pragma unroll
+                for (int r = 0; r < 8; ++r)
+                    if (own == r) from = at[r];
+                const entry_t e = uni[par][from + i];
+                // all runs' searches side by side
+                int lo[8];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) lo[r] = 0;
+#pragma unroll 1
+                for (int st = top; st > 0; st >>= 1) {
+#pragma unroll
+                    for (int r = 0; r < 8; ++r) {
+                        const int j = lo[r] + st - 1;
+                        // an empty run (or none: r >= C) reads the first entry, and nothing counts
+                        const bool below = uni[par][cn[r] > 0 ? at[r] + min(j, cn[r] - 1) : 0] < e;
+                        lo[r] += (below & (j < cn[r])) ? st : 0;
+                    }
+                }
+                int rk = 0;
+#pragma unroll
+                for (int r = 0; r < 8; ++r) rk += r == own ? i : lo[r];
+                const int p = count_below(Q, qlen, e);
+                where[rk] = p;
+                if (p + rk < L) Qn[p + rk] = e;
+            }
+            __syncthreads();
+            move_queue<NT>(Q, qlen, where, tot, Qn, L, &ctl.first_un, tid);
+            __syncthreads();
+            qlen = min(L, qlen + tot);
+            entry_t *t = Q;
+            Q = Qn;
+            Qn = t;
+        } else if (tot > 0) {
+            for (int x = tid; x < tot; x += NT) {
+                int i = x, from = at[0];
+#pragma unroll
+                for (int r = 0; r < 7; ++r)
+                    if (from == at[r] && i >= cn[r]) {
+                        i -= cn[r];
+                        from = at[r + 1];
+                    }
+                pub[x] = uni[par][from + i];
+            }
+            __syncthreads();
+            const int ncl = sort_dedupe_merge<NT>(Q, qlen, pub, tot, cand, Qn, L, any_unsafe, dup, &ctl.anydup,
+                                                  &ctl.repeats, &ctl.dropped, &ctl.first_un, tid);
             qlen = min(L, qlen + ncl);
             entry_t *t = Q;
             Q = Qn;
@@ -225,7 +301,10 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
     // distance evaluations of the whole cluster: every CTA's own fresh vertices (read before the last barrier)
     long long evals = 1;
     if (rank == 0 && tid == 0)
-        for (int r = 0; r < C; ++r) evals += *cluster.map_shared_rank(&ctl.wevals, r);
+        for (int r = 0; r < C; ++r) {
+            evals += *cluster.map_shared_rank(&ctl.wevals, r);
+            ctl.dropped += *cluster.map_shared_rank(&ctl.own_dropped, r);
+        }
     // output from rank 0 (optionally re-ranked with FP32 rows)
     if (rank == 0) {
         const entry_t *res = Q;
@@ -238,19 +317,19 @@ __global__ void __launch_bounds__(NT, 1) cluster_search_kernel(const SearchArgs 
             if (tid == 0) ctl.rr_n = 0;
             __syncthreads();
             if (!gather_fixed<ANN_STORE_F32, L2>(a.base32, nullptr, (uint32_t)a.d_pad32 / 4u, a.team_lanes32, qv,
-                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, uni, &ctl.rr_n, lane))
+                                                 cand, nullptr, qlen, warp, NW, kEmptyEntry, pub, &ctl.rr_n, lane))
                 compute_keys_teams_m<ANN_STORE_F32, NT, L2, 2>(a.base32, nullptr, a.d_pad32, qv, cand, qlen,
-                                                               a.team_lanes32, kEmptyEntry, uni, &ctl.rr_n);
+                                                               a.team_lanes32, kEmptyEntry, pub, &ctl.rr_n);
             __syncthreads();
             if (k <= 32) {
-                res = block_topk<NT>(uni, qlen, k, cand, uni);
+                res = block_topk<NT>(pub, qlen, k, cand, pub);
             } else {
                 int P = 32;
                 while (P < qlen) P <<= 1;
-                for (int i = qlen + tid; i < P; i += NT) uni[i] = kEmptyEntry;
+                for (int i = qlen + tid; i < P; i += NT) pub[i] = kEmptyEntry;
                 __syncthreads();
-                block_bitonic_sort<NT>(uni, P);
-                res = uni;
+                block_bitonic_sort<NT>(pub, P);
+                res = pub;
             }
         }
         int64_t *oid = a.out_ids + (size_t)qi * a.k;

@@ -167,6 +167,17 @@ __device__ __forceinline__ uint4 ld_row_chunk(const uint4 *p) {
     return v;
 }
 
+// The same under a predicate instead of a branch (zeros where p is false).
+__device__ __forceinline__ uint4 ld_row_chunk_if(bool pred, const uint4 *p) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.s32 p, %5, 0;\n"
+        "@p ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];\n}\n"
+        : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
+        : "l"(p), "r"((int)pred));
+    return v;
+}
+
 // Keys of the nc candidates whose ids sit in the low word of cand[0..nc).
 // A team of TS lanes (a power of two, TS >= chunks per row when the row has
 // at most 32 chunks) gathers one row with 16-byte loads; each team keeps U
@@ -785,39 +796,48 @@ __device__ __forceinline__ void warp_keys_append_m(const void *rows, const float
     const int lane = threadIdx.x & 31;
     const int ts = 1 << lts, rpw = 32 >> lts;
     const int team = lane >> lts, tl = lane & (ts - 1);
-    constexpr bool l2 = L2;
-    const uint4 *rbase = reinterpret_cast<const uint4 *>(rows);
+    const uint4 *rbase = reinterpret_cast<const uint4 *>(rows) + tl;
+    const float *qt = qv + tl * EPC;
+    const int full = (int)cpr >> lts;             // chunks that every lane of a team has
+    const bool more = (full << lts) + tl < (int)cpr;  // this lane has one more
 #pragma unroll 1
     for (int c0 = pass_begin * rpw; c0 < nf; c0 += pass_step * rpw) {
         const int c = c0 + team;
         const bool valid = c < nf;
-        const uint2 f = valid ? fr[c] : make_uint2(0u, 0u);
-        const uint32_t id = f.x;
-        const float sc = (STORE == ANN_STORE_E4M3 && valid) ? __ldg(scales + f.y) : 1.f;
+        const uint2 f = fr[valid ? c : c0];  // a team past the end re-reads a row, and its key is dropped
+        const float sc = STORE == ANN_STORE_E4M3 ? __ldg(scales + f.y) : 1.f;
         const uint4 *rp = rbase + (size_t)f.y * cpr;
         float2 acc = make_float2(0.f, 0.f);
-        if (valid) {
+        int ch = 0;
+        // whole rounds of G chunks a lane, without a test a chunk (with one, every load waited for the one before)
 #pragma unroll 1
-            for (uint32_t ch0 = tl; ch0 < cpr; ch0 += ts * G) {
-                uint4 v[G];
+        for (; ch + G <= full; ch += G) {
+            uint4 v[G];
 #pragma unroll
-                for (int g = 0; g < G; ++g)
-                    if (ch0 + g * ts < cpr) v[g] = ld_row_chunk(rp + ch0 + g * ts);
+            for (int g = 0; g < G; ++g) v[g] = ld_row_chunk(rp + ((ch + g) << lts));
 #pragma unroll
-                for (int g = 0; g < G; ++g)
-                    if (ch0 + g * ts < cpr) Chunk<STORE>::add(acc, v[g], qv + (ch0 + g * ts) * EPC, sc, l2);
-            }
+            for (int g = 0; g < G; ++g) Chunk<STORE>::add(acc, v[g], qt + ((ch + g) << lts) * EPC, sc, L2);
         }
+        // the rest: up to G - 1 chunks of every lane, and one more of some
+        uint4 v[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) v[g] = ld_row_chunk_if((ch + g < full) | ((ch + g == full) & more), rp + ((ch + g) << lts));
+#pragma unroll
+        for (int g = 0; g < G; ++g)
+            if ((ch + g < full) | ((ch + g == full) & more))
+                Chunk<STORE>::add(acc, v[g], qt + ((ch + g) << lts) * EPC, sc, L2);
         float r = acc.x + acc.y;
 #pragma unroll 1
         for (int off = ts >> 1; off > 0; off >>= 1) r += __shfl_xor_sync(kFull, r, off);
-        const entry_t e = pack_entry(l2 ? r : -r, id);
-        const bool keep = tl == 0 && valid && e < limit;
+        const entry_t e = pack_entry(L2 ? r : -r, f.x);
+        const bool keep = (tl == 0) & valid & (e < limit);
         const unsigned bal = __ballot_sync(kFull, keep);
-        int base = 0;
-        if (lane == 0 && bal) base = atomicAdd(out_n, __popc(bal));
-        base = __shfl_sync(kFull, base, 0);
-        if (keep) out[base + __popc(bal & ((1u << lane) - 1u))] = e;
+        if (bal) {
+            int base = 0;
+            if (lane == 0) base = atomicAdd(out_n, __popc(bal));
+            base = __shfl_sync(kFull, base, 0);
+            if (keep) out[base + __popc(bal & ((1u << lane) - 1u))] = e;
+        }
     }
 }
 
@@ -1216,6 +1236,34 @@ __device__ __forceinline__ int expand_step(const SearchArgs &a, uint32_t *table,
     return nf;
 }
 
+// The queued entries Q[0..qlen) to their places in Qn, up by the survivors
+// placed before them: where[r] (its low 16 bits) is the queue position of the
+// survivor of rank r, r < kept, ascending. Lowers *first_un to the first of
+// them. No barrier.
+template <int NT>
+__device__ __forceinline__ void move_queue(const entry_t *Q, int qlen, const int *where, int kept, entry_t *Qn, int L,
+                                           int *first_un, int tid) {
+    if (tid == 0 && kept > 0 && (where[0] & 0xFFFF) < *first_un) *first_un = where[0] & 0xFFFF;
+    const int per = (qlen + NT - 1) / NT, i1 = min((tid + 1) * per, qlen);
+    int i = tid * per;
+    if (i < i1) {
+        int lo = 0;  // survivors placed at or before position i
+#pragma unroll 1
+        for (int hi = kept; lo < hi;) {
+            const int mid = (lo + hi) >> 1;
+            const bool below = (where[mid] & 0xFFFF) <= i;
+            lo = below ? mid + 1 : lo;
+            hi = below ? hi : mid;
+        }
+#pragma unroll 1
+        for (; i < i1; ++i) {
+#pragma unroll 1
+            while (lo < kept && (where[lo] & 0xFFFF) <= i) ++lo;
+            if (i + lo < L) Qn[i + lo] = Q[i];
+        }
+    }
+}
+
 // The merge for few survivors (ns <= NT, one a thread), which most steps
 // have (of the 25 steps of a query at L = 576, M = 32: 13 with 32 or fewer, 18
 // with 128 or fewer): nothing is sorted. A survivor's place in the new queue is the number of
@@ -1269,25 +1317,7 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
             surv[tid] = e = kEmptyEntry;
             atomicAdd(repeats, 1);
         }
-        if (tid == 0 && kept > 0 && (where[0] & 0xFFFF) < *first_un) *first_un = where[0] & 0xFFFF;
-        const int per = (qlen + NT - 1) / NT, i1 = min((tid + 1) * per, qlen);
-        int i = tid * per;
-        if (i < i1) {
-            int lo = 0;  // survivors placed at or before position i
-#pragma unroll 1
-            for (int hi = kept; lo < hi;) {
-                const int mid = (lo + hi) >> 1;
-                const bool below = (where[mid] & 0xFFFF) <= i;
-                lo = below ? mid + 1 : lo;
-                hi = below ? hi : mid;
-            }
-#pragma unroll 1
-            for (; i < i1; ++i) {
-#pragma unroll 1
-                while (lo < kept && (where[lo] & 0xFFFF) <= i) ++lo;
-                if (i + lo < L) Qn[i + lo] = Q[i];
-            }
-        }
+        move_queue<NT>(Q, qlen, where, kept, Qn, L, first_un, tid);
         __syncthreads();
         if (!unsafe) return kept;
         const int n = *repeats;
@@ -1299,6 +1329,57 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
         }
         kept -= n;
     }
+}
+
+// Sorts in[0..n) by (key, id), n > 1 (one a thread: warp runs plus binary-search
+// ranks into `scratch`; above that warp runs merged pairwise between in and
+// `scratch`), and, with `unsafe`, drops entries whose id is queued in Q[0..qlen)
+// or repeated (counted in *dropped). Returns the sorted array and in *n what it
+// holds. dup is n bytes, *left an int in shared memory. Ends with a barrier.
+template <int NT>
+__device__ __forceinline__ entry_t *sort_dedupe(const entry_t *Q, int qlen, entry_t *in, int *n, entry_t *scratch,
+                                                bool unsafe, unsigned char *dup, int *left, long long *dropped,
+                                                int tid) {
+    const int lane = tid & 31, warp = tid >> 5, ns = *n;
+    entry_t *srt;
+    if (ns <= NT) {
+        block_rank_sort<NT>(in, ns, scratch);
+        srt = scratch;
+    } else {
+        srt = block_merge_sort<NT>(in, ns, scratch);
+    }
+    if (!unsafe) return srt;
+    int any = 0;
+#pragma unroll 1
+    for (int j = tid; j < ns; j += NT) {
+        const entry_t c = srt[j];
+        bool d = (j > 0 && srt[j - 1] == c);
+        if (!d) {
+            const int pos = count_below(Q, qlen, c);
+            d = pos < qlen && (Q[pos] & kMask) == c;
+        }
+        dup[j] = d;
+        any |= d;
+    }
+    if (__syncthreads_or(any)) {
+        if (warp == 0) {
+            int outp = 0;
+#pragma unroll 1
+            for (int b = 0; b < ns; b += 32) {
+                const int j = b + lane;
+                const bool keep = j < ns && !dup[j];
+                const entry_t c = j < ns ? srt[j] : 0ull;
+                const unsigned bal = __ballot_sync(kFull, keep);
+                if (keep) srt[outp + __popc(bal & ((1u << lane) - 1u))] = c;
+                outp += __popc(bal);
+            }
+            if (lane == 0) *left = outp;
+        }
+        __syncthreads();
+        *n = *left;
+        if (tid == 0) *dropped += ns - *n;
+    }
+    return srt;
 }
 
 // The ns (> 0) survivors in surv, in no order, are merged into the sorted
@@ -1317,50 +1398,11 @@ template <int NT>
 __device__ __forceinline__ int sort_dedupe_merge(const entry_t *Q, int qlen, entry_t *surv, int ns, entry_t *scratch,
                                                  entry_t *Qn, int L, bool unsafe, unsigned char *dup, int *anydup,
                                                  int *repeats, long long *dropped, int *first_un, int tid) {
-    const int lane = tid & 31, warp = tid >> 5;
     if (ns <= (NT < 128 ? NT : 128))
         return merge_by_rank<NT>(Q, qlen, surv, ns, reinterpret_cast<int *>(scratch), Qn, L, unsafe, repeats,
                                  dropped, first_un, tid);
-    entry_t *srt;
-    if (ns <= NT) {
-        block_rank_sort<NT>(surv, ns, scratch);
-        srt = scratch;
-    } else {
-        srt = block_merge_sort<NT>(surv, ns, scratch);
-    }
     int ncl = ns;
-    if (unsafe) {
-        int any = 0;
-#pragma unroll 1
-        for (int j = tid; j < ns; j += NT) {
-            const entry_t c = srt[j];
-            bool d = (j > 0 && srt[j - 1] == c);
-            if (!d) {
-                const int pos = count_below(Q, qlen, c);
-                d = pos < qlen && (Q[pos] & kMask) == c;
-            }
-            dup[j] = d;
-            any |= d;
-        }
-        if (__syncthreads_or(any)) {
-            if (warp == 0) {
-                int outp = 0;
-#pragma unroll 1
-                for (int b = 0; b < ns; b += 32) {
-                    const int j = b + lane;
-                    const bool keep = j < ns && !dup[j];
-                    const entry_t c = j < ns ? srt[j] : 0ull;
-                    const unsigned bal = __ballot_sync(kFull, keep);
-                    if (keep) srt[outp + __popc(bal & ((1u << lane) - 1u))] = c;
-                    outp += __popc(bal);
-                }
-                if (lane == 0) *anydup = outp;
-            }
-            __syncthreads();
-            ncl = *anydup;
-            if (tid == 0) *dropped += ns - ncl;
-        }
-    }
+    const entry_t *srt = sort_dedupe<NT>(Q, qlen, surv, &ncl, scratch, unsafe, dup, anydup, dropped, tid);
     // the first survivor's rank among the old entries bounds the new queue's checked prefix
     if (tid == 0 && ncl > 0) {
         const int p0 = count_below(Q, qlen, srt[0]);

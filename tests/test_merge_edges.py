@@ -59,3 +59,25 @@ def test_prefetch_lines_cover_a_row():
             touched = set(range(p // 128, (p + row_bytes - 1) // 128 + 1))
             asked = {(p + 128 * i) // 128 for i in range(lines - 1)} | {(p + row_bytes - 1) // 128}
             assert touched <= asked and len(asked - touched) == 0, (row_bytes, row)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("C", [2, 4, 8])
+@pytest.mark.parametrize("hash_bits", [0, 8])
+def test_one_cta_of_a_cluster_owns_every_vertex(oracle_mod, C, hash_bits):
+    """Only ids that are multiples of 8 are reachable: one CTA finds every survivor, more than its share of the
+    exchange buffers, in steps with few and with many of them."""
+    from paper_2201_13007_gb300.index import Index
+    g = np.random.Generator(np.random.PCG64(2))
+    m, R, d = 3000, 32, 32
+    n = 8 * m
+    base = g.integers(0, 256, (n, d)).astype(np.float32)
+    adj = np.full((n, R), -1, np.int32)
+    adj[::8] = 8 * g.integers(0, m, (m, R))
+    q = g.integers(0, 256, (6, d)).astype(np.float32)
+    ix = Index(base, adj, 0)
+    for L, M in ((40, 8), (300, 16), (600, 64)):
+        o_ids, o_keys, _ = oracle_mod.search(base, adj, 0, q, algo="topm", L=L, K=10, M0=1, M_max=M, t=1, nthreads=8)
+        ids, dists = ix.search(torch.from_numpy(q).cuda(), 10, L, M, cluster=C, hash_bits=hash_bits)
+        compare_exact(ids.cpu().numpy(), dists.cpu().numpy(), o_ids, o_keys)
+    ix.close()
