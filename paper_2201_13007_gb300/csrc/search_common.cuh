@@ -861,8 +861,8 @@ __device__ __forceinline__ void warp_keys_fixed(const void *rows, const float *s
     const float *qt = qv + tl * EPC;
     // Two passes at once while there are that many: their loads are in flight together and share the query's chunks
     // (a step's gather at L = 576, M = 32, four CTAs of 256 threads per SM: 14,600 cycles with one, 10,900 with two;
-    // 1,000 queries of 960-d FP16 rows: 4.44 and 4.00 ms). FP32 rows fill the registers with one (two spill: 12.2 ms
-    // against 9.6 for 10,000 queries).
+    // 1,000 queries of 960-d FP16 rows: 4.44 and 4.00 ms). FP32 rows have twice the chunks: one pass, all of a 128-d
+    // row's loads in flight (10,000 queries: 7.91 ms with half of them in flight, 7.74 with all; two passes spill, 12.2).
     auto pass = [&](auto u_, int c0) {
         constexpr int U = decltype(u_)::value;
         uint32_t id[U];
@@ -953,10 +953,10 @@ __device__ __forceinline__ bool gather_fixed(const void *rows, const float *scal
         ANN_FIXED(2, 3, 3)   // 96-d
         ANN_FIXED(3, 15, 5)  // 960-d
     } else if constexpr (STORE == ANN_STORE_F32) {
-        ANN_FIXED(2, 8, 4)   // 128-d
-        ANN_FIXED(2, 6, 3)   // 96-d
+        ANN_FIXED(2, 8, 8)   // 128-d
+        ANN_FIXED(2, 6, 6)   // 96-d
         ANN_FIXED(2, 2, 2)   // 32-d
-        ANN_FIXED(3, 30, 5)  // 960-d
+        ANN_FIXED(3, 30, 6)  // 960-d
     } else {
         ANN_FIXED(2, 15, 5)  // 960-d
         ANN_FIXED(2, 2, 2)   // 128-d

@@ -81,3 +81,18 @@ def test_one_cta_of_a_cluster_owns_every_vertex(oracle_mod, C, hash_bits):
         ids, dists = ix.search(torch.from_numpy(q).cuda(), 10, L, M, cluster=C, hash_bits=hash_bits)
         compare_exact(ids.cpu().numpy(), dists.cpu().numpy(), o_ids, o_keys)
     ix.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("L,M", [(40, 32), (300, 16), (700, 64), (1500, 48)])
+def test_wide_first_steps(env, oracle_mod, L, M):
+    """M from the first step on: hundreds of survivors meet a queue of a few dozen, so that many fall between the same
+    two entries, and a queue that overflows at once."""
+    base, w, ix = env
+    q = torch.from_numpy(w.queries).cuda()
+    o_ids, o_keys, _ = oracle_mod.search(base, w.adj, w.entry, w.queries, algo="topm", L=L, K=10, M0=M, M_max=M, t=1,
+                                         nthreads=8)
+    for threads, cluster in ((64, 1), (128, 1), (256, 1), (512, 1), (256, 4)):
+        for hash_bits in (8, 13):
+            ids, d = ix.search(q, 10, L, M, M0=M, threads=threads, hash_bits=hash_bits, cluster=cluster, visited_mode=4)
+            compare_exact(ids.cpu().numpy(), d.cpu().numpy(), o_ids, o_keys)
