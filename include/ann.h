@@ -253,7 +253,8 @@ int ann_index_group_neighbors(ann_index *index, float hot_fraction, int32_t pref
  * alignment, range), ANN_ERR_OOM, ANN_ERR_CUDA. Work: n * nq * d
  * multiply-adds on the tensor cores. The call allocates device memory and
  * frees it before it returns: 36 bytes per base row and up to 3 KB per query
- * of a chunk of 58,000 (8 KB while fewer than 29,000, 16 KB below 15,000). */
+ * of a chunk of 58,000 (5 KB while fewer than 29,000, 9 KB below 15,000); with
+ * no room for that, 4 bytes per base row, and the call is slower. */
 int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, int64_t nq, int64_t self_offset,
                  int32_t metric, int32_t k, int32_t *out_ids, float *out_dists, void *stream);
 

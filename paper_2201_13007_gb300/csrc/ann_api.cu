@@ -582,12 +582,19 @@ int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, in
     const int sms = sm_count();
     const ann::KnnPlan plan = ann::knn_plan(n, nq, sms);
     unsigned char *ws = nullptr;
-    cudaError_t e;
-    if ((e = cudaMalloc(&ws, plan.bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc(knn workspace)");
+    size_t err_at = plan.err;
+    cudaError_t e = cudaMalloc(&ws, plan.bytes);
+    const bool scan = e == cudaErrorMemoryAllocation;  // no room for the filter's lists: 4 bytes a base row will do
+    if (scan) {
+        cudaGetLastError();
+        err_at = 0;
+        e = cudaMalloc(&ws, ann::knn_scan_bytes(n));
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(knn workspace)");
     int herr = 0;
-    if ((e = ann::launch_knn_bf16(plan, ws, base, n, d, queries, nq, self_offset, metric, k, out_ids, out_dists, sms,
-                                  s)) == cudaSuccess &&
-        (e = cudaMemcpyAsync(&herr, ws + plan.err, 4, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
+    e = scan ? ann::launch_knn_scan_all(ws, base, n, d, queries, nq, self_offset, metric, k, out_ids, out_dists, s)
+             : ann::launch_knn_bf16(plan, ws, base, n, d, queries, nq, self_offset, metric, k, out_ids, out_dists, sms, s);
+    if (e == cudaSuccess && (e = cudaMemcpyAsync(&herr, ws + err_at, 4, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
         e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) cudaStreamSynchronize(s);  // nothing may use the workspace when it is freed
     cudaFree(ws);

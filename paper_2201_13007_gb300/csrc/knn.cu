@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(KNT, 1)
                     const __nv_bfloat16 *__restrict__ queries, int64_t nq, int64_t self0, int k,
                     int32_t *__restrict__ out_ids, float *__restrict__ out_d, const int *__restrict__ only,
                     int *__restrict__ err) {
-    if (!only[blockIdx.x]) return;
+    if (only && !only[blockIdx.x]) return;
     constexpr int D = KS * 16;
     constexpr int P = knn_pitch(D);
     constexpr int CPR = D / 8;  // 16-byte chunks per row

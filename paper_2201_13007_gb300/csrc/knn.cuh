@@ -19,8 +19,13 @@ KnnPlan knn_plan(int64_t n, int64_t nq, int sms);
 cudaError_t launch_knn_bf16(const KnnPlan &plan, void *ws, const void *base, int64_t n, int d, const void *queries,
                             int64_t nq, int64_t self0, int metric, int k, int32_t *ids, float *dists, int sms,
                             cudaStream_t stream);
+// The same by the scan kernel alone, for callers without room for the plan's
+// workspace: ws holds knn_scan_bytes(n); its first int is the error word.
+size_t knn_scan_bytes(int64_t n);
+cudaError_t launch_knn_scan_all(void *ws, const void *base, int64_t n, int d, const void *queries, int64_t nq,
+                                int64_t self0, int metric, int k, int32_t *ids, float *dists, cudaStream_t stream);
 // knn.cu: the scan kernel, for the blocks of 128 query rows with only[block]
-// set. norms holds the base rows' squared norms (zeros up to
+// set (all if only is null). norms holds the base rows' squared norms (zeros up to
 // knn_norms_rows(n)); err is set to 1 if a CTA's merge rounds ran out.
 int64_t knn_norms_rows(int64_t n);
 cudaError_t launch_knn_scan(const void *base, int64_t n, int d, const void *queries, int64_t nq, int64_t self0,

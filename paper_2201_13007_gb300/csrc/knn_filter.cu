@@ -439,8 +439,8 @@ __host__ __device__ inline int64_t segment_row0(int64_t n, int levels, int s) {
 
 // ---------------------------------------------------------------- rows
 // Norms of the base rows in order (as the scan kernel wants them: zeros up to
-// n_pad), the bias rows (-|x|^2 / 2, or 0) in segment order, and the largest
-// norm (its bits).
+// n_pad), the bias rows (-|x|^2 / 2, or 0; none if bias is null) in segment
+// order, and the largest norm (its bits).
 __global__ void knn_base_rows(const __nv_bfloat16 *__restrict__ x, int64_t n, int64_t n_pad, int d, int levels, bool l2,
                               float *__restrict__ norms, unsigned char *__restrict__ bias,
                               unsigned *__restrict__ top) {
@@ -452,14 +452,16 @@ __global__ void knn_base_rows(const __nv_bfloat16 *__restrict__ x, int64_t n, in
         const int low = i == 0 ? levels : min(levels, __ffsll(i) - 1);
         const int64_t at = low == levels ? i >> levels
                                          : segment_row0(n, levels, levels - low) + (i >> (low + 1));
-        const float b = l2 ? -0.5f * nrm : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(b);
-        const float r = b - __bfloat162float(h);
-        const __nv_bfloat16 m = __float2bfloat16_rn(r);
-        const __nv_bfloat16 l = __float2bfloat16_rn(r - __bfloat162float(m));
-        const uint4 part = make_uint4((uint32_t)__bfloat16_as_ushort(h) | (uint32_t)__bfloat16_as_ushort(m) << 16,
-                                      (uint32_t)__bfloat16_as_ushort(l), 0u, 0u);
-        *reinterpret_cast<uint4 *>(bias + at / FN * (FN * kBiasRow) + at % FN * 16) = part;
+        if (bias) {
+            const float b = l2 ? -0.5f * nrm : 0.f;
+            const __nv_bfloat16 h = __float2bfloat16_rn(b);
+            const float r = b - __bfloat162float(h);
+            const __nv_bfloat16 m = __float2bfloat16_rn(r);
+            const __nv_bfloat16 l = __float2bfloat16_rn(r - __bfloat162float(m));
+            const uint4 part = make_uint4((uint32_t)__bfloat16_as_ushort(h) | (uint32_t)__bfloat16_as_ushort(m) << 16,
+                                          (uint32_t)__bfloat16_as_ushort(l), 0u, 0u);
+            *reinterpret_cast<uint4 *>(bias + at / FN * (FN * kBiasRow) + at % FN * 16) = part;
+        }
     }
     if (i < n_pad) norms[i] = nrm;
     unsigned m = __float_as_uint(nrm);  // not finite: above every finite value
@@ -754,6 +756,23 @@ cudaError_t launch_finish(const void *base, const float *norms, const void *q, c
 }
 
 }  // namespace
+
+size_t knn_scan_bytes(int64_t n) { return 256 + (size_t)knn_norms_rows(n) * 4; }
+
+cudaError_t launch_knn_scan_all(void *ws, const void *base, int64_t n, int d, const void *queries, int64_t nq,
+                                int64_t self0, int metric, int k, int32_t *ids, float *dists, cudaStream_t s) {
+    unsigned char *w = static_cast<unsigned char *>(ws);
+    float *norms = reinterpret_cast<float *>(w + 256);
+    const int64_t np = knn_norms_rows(n);
+    cudaError_t e = cudaMemsetAsync(w, 0, 256, s);
+    if (e != cudaSuccess) return e;
+    knn_base_rows<<<(unsigned)((np + 255) / 256), 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(base), n, np, d, 0,
+                                                               metric == ANN_METRIC_L2, norms, nullptr,
+                                                               reinterpret_cast<unsigned *>(w + 4));
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_knn_scan(base, n, d, queries, nq, self0, metric, k, ids, dists, norms, nullptr,
+                           reinterpret_cast<int *>(w), s);
+}
 
 KnnPlan knn_plan(int64_t n, int64_t nq, int sms) {
     KnnPlan p;

@@ -83,3 +83,21 @@ def test_not_finite_rows_return():
     base, bits = _bf16(x)
     gi, gd = _gpu_knn(bits, bits[:300], 0, "l2", 8)
     assert gi.shape == (300, 8) and ((gi >= -1) & (gi < 1500)).all()
+
+
+@pytest.mark.gpu
+def test_without_room_for_the_lists():
+    """With too little free device memory for the filter's lists (201 MB here) the scan kernel answers alone: the same
+    bits."""
+    import torch
+    _, bits = _bf16(_integer_rows(3000, 32, 4))
+    ref = _gpu_knn(bits, bits, 0, "l2", 20)
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    hold = torch.empty(free - (96 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = _gpu_knn(bits, bits, 0, "l2", 20)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(ref[0], got[0]) and np.array_equal(ref[1], got[1])
