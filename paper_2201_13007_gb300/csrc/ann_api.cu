@@ -213,22 +213,24 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     if (p->merge_rule == 1 && !(p->patience >= 0.f))
         return fail(ANN_ERR_ARG, "patience must be >= 0 (or INFINITY) with merge_rule 1");
     if (async && M > 32) return fail(ANN_ERR_ARG, "async mode runs one warp per walker: M=%d > 32", M);
-    // cluster = 0: while the SMs allow it each query runs on a cluster of CTAs, when the cluster kernel runs the search
-    // as asked (sync, not persistent, no phase counters, no neighbour groups, a set-associative visited set); the
-    // results are those of one CTA per query. If that plan does not fit, one CTA per query. The lines: a cluster of 8
-    // needs 8 free SMs of one GPC, and from 16 queries on they no longer all run at once (100 x 8 searches of 96-d
-    // BF16 rows, us, clusters of 8 / 4 / 2 / one CTA: 9 queries 114 / 115 / 120 / 132, 16: 195 / 116 / 122 / 134, 32:
-    // - / 133 / 141 / 151, 64: - / 232 / 144 / 155, 128: - / - / 257 / 164).
-    if (p->cluster == 0 && nq >= 1 && !async && !p->persistent && !p->phase_cycles &&
-        (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0) {
-        const int sms = sm_count();
-        const int c = 12 * nq <= sms || (nq <= 8 && 8 * nq <= sms) ? 8 : 9 * nq <= 2 * sms ? 4 : 2 * nq <= sms ? 2 : 1;
-        if (c > 1) {
+    // cluster = 0, at most 8 queries and steps that gather 96 KB of rows or more: each query on a cluster of 8 CTAs (4,
+    // 2 if fewer SMs), when the cluster kernel runs the search as asked (sync, not persistent, no phase counters, no
+    // neighbour groups, a set-associative visited set); the results are those of one CTA per query. If that plan does
+    // not fit, one CTA per query. The lines, us for one query (and for eight), 8 CTAs against one: 96-d BF16 rows, M = 8
+    // (48 KB) 107 / 98 (109 / 98), M = 16 (96 KB) 112 / 116 (124 / 126), M = 32 156 / 167 (181 / 201); 128-d FP32, M = 32
+    // 90 / 110 (101 / 127); 960-d FP8, M = 8 165 / 193 (eight). Above eight queries a cluster gains nothing alone (33
+    // queries, M = 16: 128 / 127) and takes the SMs of calls on other streams (six streams of them: 555 / 248).
+    if (p->cluster == 0 && nq >= 1 && nq <= 8 && !async && !p->persistent && !p->phase_cycles &&
+        (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0 &&
+        (int64_t)M * x.R * x.d_pad * ann::storage_bytes(x.storage) >= (96 << 10)) {
+        for (int c = 8; c >= 2; c >>= 1) {
+            if ((int64_t)nq * c > sm_count()) continue;
             ann_search_params pc = *p;
             pc.cluster = c;
             const std::string saved = g_err;
             if (plan_search(index, queries, nq, k, L, M, out_ids, out_dists, &pc, plan) == ANN_OK) return ANN_OK;
             g_err = saved;
+            break;
         }
     }
     const int csize = p->cluster > 1 ? p->cluster : 1;
@@ -236,14 +238,16 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
         return fail(ANN_ERR_ARG, "cluster=%d not in {0, 1, 2, 4, 8}", p->cluster);
     if (csize > 1 && async) return fail(ANN_ERR_ARG, "clusters are for sync mode only");
     int threads = p->threads;
-    // Automatic launch shape of the one-CTA sync kernel, from sweeps of threads and visited bits over 152 to 10,000
-    // queries (1M x 96 BF16 and 128 FP32 rows, 200,000 x 960 FP16 and FP8 rows). An SM holds 1,024 threads of it, so
-    // with up to two queries per SM each takes 512 threads (256 if its steps have fewer than 256 slots), with up to
-    // four 256, and a visited set that lets them all reside. Beyond that throughput counts: 256 threads for steps of
-    // 1,024 slots or more, 512 where such steps would gather 768 KB of rows over 1 KB, else 128 or 256, whichever
-    // needs less time for its rounds of resident queries (a round of 128-thread CTAs takes 1.3 times one of 256).
-    // Against the former line at 32 queries per SM (us): 256 queries, L = 192, M = 16 290 -> 190; 456, L = 576, M = 32
-    // 508 -> 393; 2,432, L = 1024, M = 4 12,254 -> 5,771; 1,000 x 960-d FP8, L = 128, M = 8 1,107 -> 851.
+    // Automatic launch shape of the one-CTA sync kernel, from sweeps of threads and visited bits over 1 to 10,000
+    // queries (1M x 96 BF16 and 128 FP32 rows, 200,000 x 960 FP16 and FP8 rows). An SM holds 1,024 threads of it. Up to
+    // four queries per SM each takes 256 threads, or 512, while there are no more than two, for steps that gather 384 KB
+    // of rows, or while there is no more than one for steps of 1,024 slots (512 / 256 threads, 152 queries, us: 128-d
+    // FP32, M = 32 158 / 184, 96-d BF16, M = 32 220 / 237, M = 16 153 / 152, M = 4 129 / 119; 304 queries: 204 / 242,
+    // 264 / 253, 167 / 158, 140 / 125), and a visited set that lets them all reside. Beyond that throughput counts: 256
+    // threads for steps of 1,024 slots or more, 512 where such steps would gather 768 KB of rows over 1 KB, else 128 or
+    // 256, whichever needs less time for its rounds of resident queries (a round of 128-thread CTAs takes 1.3 times one
+    // of 256). Against the former line at 32 queries per SM (us): 256 queries, L = 192, M = 16 290 -> 190; 456, L = 576,
+    // M = 32 508 -> 393; 2,432, L = 1024, M = 4 12,254 -> 5,771; 1,000 x 960-d FP8, L = 128, M = 8 1,107 -> 851.
     const bool one = !async && csize == 1;
     const int64_t sms = sm_count(), slots = (int64_t)M * x.R;
     const int64_t row_bytes = (int64_t)x.d_pad * ann::storage_bytes(x.storage);
@@ -259,14 +263,13 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
             return fail(ANN_ERR_ARG, "threads=%d not in {64,...,1024}", threads);
         if (threads / 32 < M) return fail(ANN_ERR_ARG, "async mode needs threads >= 32*M");
     } else {
-        // clusters: 512 threads for wide steps or heavy rows, 256 for steps of 256 slots or long queues, else 128 (clusters
-        // of 8, 512 / 256 / 128 threads, us: L = 576, M = 64 122 / 132 / -, L = 576, M = 32 156 / 157 / -, L = 192, M = 16
-        // 128 / 115 / -, L = 1024, M = 4 1104 / 1020 / 1072)
-        if (threads == 0 && !one)
-            threads = slots >= 2048 || slots * row_bytes >= (512 << 10) ? 512 : (slots >= 256 || L >= 384 ? 256 : 128);
+        // clusters: 512 threads for steps of 2,048 slots, 256 for steps of 256 slots or long queues, else 128 (clusters
+        // of 8, 512 / 256 / 128 threads, us: 128-d FP32 L = 576, M = 64 138 / 150 / 192, M = 32 172 / 177 / 216; 96-d BF16
+        // L = 192, M = 16 119 / 112 / 124, L = 1024, M = 4 996 / 912 / 934; 960-d FP16 L = 768, M = 16 455 / 422 / 480)
+        if (threads == 0 && !one) threads = slots >= 2048 ? 512 : (slots >= 256 || L >= 384 ? 256 : 128);
         if (threads == 0) {
             if (few) {
-                threads = slots >= 256 ? 512 : 256;
+                threads = slots * row_bytes >= (384 << 10) || (nq <= sms && slots >= 1024) ? 512 : 256;
             } else if (long_rows) {
                 threads = 512;
             } else if (nq <= 4 * sms || slots >= 1024) {

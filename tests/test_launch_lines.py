@@ -1,5 +1,5 @@
-"""Both sides of every line of the automatic launch shape (clusters of 8, 4 and
-2 CTAs, one CTA of 512, 256 or 128 threads): the answers are those of one
+"""Both sides of every line of the automatic launch shape (clusters of 8
+CTAs, one CTA of 512, 256 or 128 threads): the answers are those of one
 explicitly shaped launch, and each side takes the shape it is meant to."""
 import pytest
 
@@ -7,12 +7,14 @@ torch = pytest.importorskip("torch")
 
 from paper_2201_13007_gb300 import synth  # noqa: E402
 
-# (queries, L, M) and the automatic (CTAs per query, threads) on a GPU of 152 SMs
+# (queries, L, M) and the automatic (CTAs per query, threads) over 128-d FP32 and BF16 rows (512 and 256 bytes, 32 to a
+# vertex) on a GPU of 152 SMs
 LINES = [
-    ((12, 100, 8), (8, 256)), ((13, 100, 8), (4, 256)), ((33, 100, 8), (4, 256)), ((34, 100, 8), (2, 256)),
-    ((76, 48, 4), (2, 128)), ((77, 48, 4), (1, 256)), ((304, 100, 8), (1, 512)), ((305, 100, 8), (1, 256)),
-    ((608, 100, 8), (1, 256)), ((609, 100, 8), (1, 128)), ((609, 100, 32), (1, 256)), ((1300, 400, 8), (1, 128)),
-    ((1000, 1024, 8), (1, 256)),
+    ((1, 48, 4), (1, 256), (1, 256)), ((8, 100, 6), (8, 128), (1, 256)), ((8, 100, 12), (8, 256), (8, 256)),
+    ((8, 100, 64), (8, 512), (8, 512)), ((9, 100, 64), (1, 512), (1, 512)), ((152, 100, 32), (1, 512), (1, 512)),
+    ((153, 100, 32), (1, 512), (1, 256)), ((304, 100, 24), (1, 512), (1, 256)), ((305, 100, 24), (1, 256), (1, 256)),
+    ((608, 100, 8), (1, 256), (1, 256)), ((609, 100, 8), (1, 128), (1, 128)), ((609, 100, 32), (1, 256), (1, 256)),
+    ((1000, 1024, 8), (1, 256), (1, 256)), ((1300, 400, 8), (1, 128), (1, 128)),
 ]
 
 
@@ -24,7 +26,8 @@ def test_every_launch_shape_gives_the_same_answers(storage):
     ix = Index(w.base, w.adj, w.entry, storage=storage, keep_f32=storage != "f32")
     q = torch.from_numpy(w.queries).cuda()
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    for (nq, L, M), shape in LINES:
+    for (nq, L, M), *shapes in LINES:
+        shape = shapes[storage == "bf16"]
         d = ix.describe(nq, 10, L, M)
         if sms == 152:
             assert (d["cluster"], d["threads"]) == shape, (nq, L, M, d)
