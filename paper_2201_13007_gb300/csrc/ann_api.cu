@@ -191,7 +191,7 @@ int create_impl(const float *base, int64_t n, int32_t d, int32_t storage, const 
 namespace ann {
 
 int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_t k, int32_t L, int32_t M,
-                int64_t *out_ids, float *out_dists, const ann_search_params *p, Plan *plan) {
+                int64_t *out_ids, float *out_dists, const ann_search_params *p, Plan *plan, int64_t together) {
     if (!index) return fail(ANN_ERR_ARG, "index is NULL");
     const ann::IndexData &x = index->d;
     if (nq < 0 || nq > 0x7fffffffll) return fail(ANN_ERR_ARG, "nq=%lld outside [0, 2^31)", (long long)nq);
@@ -251,7 +251,8 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     const bool one = !async && csize == 1;
     const int64_t sms = sm_count(), slots = (int64_t)M * x.R;
     const int64_t row_bytes = (int64_t)x.d_pad * ann::storage_bytes(x.storage);
-    const bool few = nq <= 2 * sms;
+    const int64_t load = std::max(nq, together);
+    const bool few = load <= 2 * sms;
     const bool long_rows = row_bytes > 1024 && slots * row_bytes >= (768 << 10);
     const bool heavy = L >= 384 || slots * row_bytes >= (256 << 10);  // long queues or heavy steps
     if (async) {
@@ -269,10 +270,10 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
         if (threads == 0 && !one) threads = slots >= 2048 ? 512 : (slots >= 256 || L >= 384 ? 256 : 128);
         if (threads == 0) {
             if (few) {
-                threads = slots * row_bytes >= (384 << 10) || (nq <= sms && slots >= 1024) ? 512 : 256;
+                threads = slots * row_bytes >= (384 << 10) || (load <= sms && slots >= 1024) ? 512 : 256;
             } else if (long_rows) {
                 threads = 512;
-            } else if (nq <= 4 * sms || slots >= 1024) {
+            } else if (load <= 4 * sms || slots >= 1024) {
                 threads = 256;
             } else {
                 // queries resident per SM: 1,024 threads' worth, or what shared memory holds (queues, candidate
@@ -281,7 +282,7 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
                                      1536;
                 const int64_t fit = std::max<int64_t>(1, (228 << 10) / smem);
                 const int64_t r128 = std::min<int64_t>(8, fit) * sms, r256 = std::min<int64_t>(4, fit) * sms;
-                threads = 13 * ((nq + r128 - 1) / r128) <= 10 * ((nq + r256 - 1) / r256) ? 128 : 256;
+                threads = 13 * ((load + r128 - 1) / r128) <= 10 * ((load + r256 - 1) / r256) ? 128 : 256;
             }
         }
         if (threads != 64 && threads != 128 && threads != 256 && threads != 512)
@@ -322,7 +323,7 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     };
     int hb = p->hash_bits;
     if (hb == 0) {
-        const bool packed = vmode >= 3 ? one && !few && !long_rows : one && nq >= 32 * sms;
+        const bool packed = vmode >= 3 ? one && !few && !long_rows : one && load >= 32 * sms;
         if (packed) {  // the most slots that fit in 16 KB (2^12 full ids or set words; 2^14 one-byte tags)
             hb = 12;
             for (int b = 14; b > 12; --b)

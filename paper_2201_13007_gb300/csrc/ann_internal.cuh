@@ -167,7 +167,8 @@ void set_error(const char *msg);
 // more than any earlier one (the call costs microseconds on a latency path).
 cudaError_t ensure_dyn_smem(const void *kernel, int smem);
 
-// ann_api.cu: argument checks and launch configuration of one search
+// ann_api.cu: argument checks and launch configuration of one search. together: how many queries run at the same time,
+// which the automatic launch shape goes by (0: the nq of this search; a batch gives the queries of all its launches)
 struct Plan {
     SearchArgs a;
     int threads;
@@ -178,7 +179,7 @@ struct Plan {
     int cluster;  // CTAs per query (1 = no cluster)
 };
 int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_t k, int32_t L, int32_t M,
-                int64_t *out_ids, float *out_dists, const ann_search_params *p, Plan *plan);
+                int64_t *out_ids, float *out_dists, const ann_search_params *p, Plan *plan, int64_t together = 0);
 cudaError_t launch(const Plan &plan, cudaStream_t s);
 int index_device(const ann_index *index);
 

@@ -2,10 +2,10 @@
 //
 // The planner groups queries into buckets by L, orders each bucket by
 // descending L (longest first, so a persistent grid does not end on one
-// long query) and prepares one persistent launch per bucket, whose shared
-// memory, block size and visited table are sized for that bucket only. A
-// search forks the caller's stream into one stream per bucket (event
-// record / wait), resets each bucket's work counter, launches, and joins
+// long query) and prepares one or two persistent launches per bucket, whose
+// shared memory, block size and visited table are sized for their queries
+// only. A search forks the caller's stream into one stream per launch (event
+// record / wait), resets each launch's work counter, launches, and joins
 // back: all stream-ordered, no allocation, no host synchronisation, so the
 // whole call can be captured into a CUDA graph and replayed.
 #include <algorithm>
@@ -17,7 +17,10 @@
 
 namespace {
 
-struct Bucket {
+// Queries whose steps have at most this many slots (M times R) are launched apart from the rest of their bucket
+constexpr int64_t kLightSlots = 256;
+
+struct Launch {  // a bucket, or its queries of few slots a step, or the others
     ann::Plan plan;
     int count = 0;
     int offset = 0;
@@ -38,15 +41,16 @@ struct ann_batch {
     int32_t kmax = 0;
     int32_t *d_kLM = nullptr;   // k[nq], L[nq], M[nq]
     int32_t *d_order = nullptr; // bucket work lists back to back
-    int *d_counters = nullptr;  // one per bucket
+    int *d_counters = nullptr;  // one per launch
     cudaEvent_t fork = nullptr;
-    std::vector<Bucket> buckets;
+    std::vector<Launch> launches;
+    int32_t n_buckets = 0;
 };
 
 namespace {
 
 void free_batch(ann_batch *b) {
-    for (Bucket &k : b->buckets) {
+    for (Launch &k : b->launches) {
         if (k.joined) cudaEventDestroy(k.joined);
         if (k.stream) cudaStreamDestroy(k.stream);
     }
@@ -109,8 +113,26 @@ int ann_batch_create(const ann_index *index, int64_t nq, const int32_t *k, const
         cost[i] = ((float)L[i] / (float)M[i] + 10.f) * (1.f + (float)M[i] * (float)info.R / 1024.f);
     std::vector<int32_t> order(nq);
     for (int64_t i = 0; i < nq; ++i) order[i] = (int32_t)i;
+    ann_search_params base;
+    memset(&base, 0, sizeof(base));
+    if (params) base = *params;
+    // With more than 32 queries per SM, a bucket of automatic shape is two launches: queries of few slots a step need
+    // less shared memory than the others and run best in CTAs of 128 threads. One launch a bucket / two, us, 96-d BF16
+    // rows, R = 32, the values of L and M evenly: 20,000 queries, L 32 to 1024, M 4 to 32 9,990 / 9,230; 8,000 of them
+    // 4,115 / 3,960; 5,000, L 512 and 1024, M 1, 2 and 32 14,430 / 10,190; 10,000, L = 576, M 8 and 12 5,515 / 5,400. With
+    // fewer the rounds of the two parts do not even out (2,500, L = 1024, M 8 and 16 2,936 / 3,108), and with M = 16 among
+    // the light ones batches of M 16 and 32 lose (5,000, L 100 and 200 1,071 / 1,129).
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    auto splits = [&](int b) {
+        return base.mode == ANN_MODE_SYNC && !base.threads && !cfg[b].threads && nq > 32 * (int64_t)sms;
+    };
+    std::vector<char> light(nq);
+    for (int64_t i = 0; i < nq; ++i) light[i] = splits(which[i]) && (int64_t)M[i] * info.R <= kLightSlots;
     std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
         if (which[a] != which[b]) return which[a] < which[b];
+        if (light[a] != light[b]) return light[a] < light[b];
         return cost[a] > cost[b];
     });
     std::vector<int32_t> kLM(3 * nq);
@@ -119,7 +141,7 @@ int ann_batch_create(const ann_index *index, int64_t nq, const int32_t *k, const
     memcpy(kLM.data() + 2 * nq, M, nq * 4);
     cudaError_t e = cudaMalloc(&bt->d_kLM, 3 * nq * 4);
     if (e == cudaSuccess) e = cudaMalloc(&bt->d_order, nq * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&bt->d_counters, cfg.size() * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&bt->d_counters, 2 * cfg.size() * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(bt->d_kLM, kLM.data(), 3 * nq * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(bt->d_order, order.data(), nq * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bt->fork, cudaEventDisableTiming);
@@ -128,20 +150,18 @@ int ann_batch_create(const ann_index *index, int64_t nq, const int32_t *k, const
         cudaGetLastError();
         return bfail(e == cudaErrorMemoryAllocation ? ANN_ERR_OOM : ANN_ERR_CUDA, cudaGetErrorString(e));
     }
-    ann_search_params base;
-    memset(&base, 0, sizeof(base));
-    if (params) base = *params;
     int64_t pos = 0;
-    for (int b = 0; b < (int)cfg.size(); ++b) {
+    for (int at = 0; at < 2 * (int)cfg.size(); ++at) {
+        const int b = at / 2, part = at & 1;
         int64_t n = 0;
         int32_t Lm = 0, Mm = 0;
-        while (pos + n < nq && which[order[pos + n]] == b) {
+        while (pos + n < nq && which[order[pos + n]] == b && light[order[pos + n]] == part) {
             Lm = std::max(Lm, L[order[pos + n]]);
             Mm = std::max(Mm, M[order[pos + n]]);
             n++;
         }
         if (n == 0) continue;
-        Bucket bk;
+        Launch bk;
         bk.count = (int)n;
         bk.offset = (int)pos;
         ann_search_params p = base;
@@ -153,17 +173,31 @@ int ann_batch_create(const ann_index *index, int64_t nq, const int32_t *k, const
         if (cfg[b].threads) p.threads = cfg[b].threads;
         if (cfg[b].hash_bits) p.hash_bits = cfg[b].hash_bits;
         // device pointers for queries / outputs are bound at search time
-        int rc = ann::plan_search(index, reinterpret_cast<const float *>(16), n, std::min(kmax, Lm), Lm, Mm,
-                                  reinterpret_cast<int64_t *>(16), reinterpret_cast<float *>(16), &p, &bk.plan);
+        auto plan = [&](int32_t Lp, int32_t Mp) {
+            return ann::plan_search(index, reinterpret_cast<const float *>(16), n, std::min(kmax, Lp), Lp, Mp,
+                                    reinterpret_cast<int64_t *>(16), reinterpret_cast<float *>(16), &p, &bk.plan, splits(b) ? nq : 0);
+        };
+        int rc = ANN_OK;
+        if (part == 0 || pos == 0 || which[order[pos - 1]] != b) {  // the bucket's first launch
+            ++bt->n_buckets;
+            int32_t La = Lm, Ma = Mm;
+            for (int64_t i = pos + n; i < nq && which[order[i]] == b; ++i) {
+                La = std::max(La, L[order[i]]);
+                Ma = std::max(Ma, M[order[i]]);
+            }
+            // a bucket too large for one launch is refused, whether or not its parts would fit
+            if (La > Lm || Ma > Mm) rc = plan(La, Ma);
+        }
+        if (rc == ANN_OK) rc = plan(Lm, Mm);
         if (rc != ANN_OK) {
             free_batch(bt);
             return rc;
         }
         bk.plan.a.k = kmax;  // output row stride (and per-query k bound) of the whole batch
-        bk.plan.a.work_counter = bt->d_counters + bt->buckets.size();
+        bk.plan.a.work_counter = bt->d_counters + bt->launches.size();
         e = cudaStreamCreateWithFlags(&bk.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bk.joined, cudaEventDisableTiming);
-        bt->buckets.push_back(bk);
+        bt->launches.push_back(bk);
         if (e != cudaSuccess) {
             free_batch(bt);
             return bfail(ANN_ERR_CUDA, cudaGetErrorString(e));
@@ -183,8 +217,8 @@ int ann_batch_search(ann_batch *bt, const float *queries, int64_t *out_ids, floa
     cudaError_t e = cudaEventRecord(bt->fork, s);
     // the buckets with the longest queues first: whatever is launched first takes the SMs first, and a long query that
     // starts late ends late
-    for (size_t b = bt->buckets.size(); e == cudaSuccess && b-- > 0;) {
-        Bucket &bk = bt->buckets[b];
+    for (size_t b = bt->launches.size(); e == cudaSuccess && b-- > 0;) {
+        Launch &bk = bt->launches[b];
         bk.plan.a.queries = queries;
         bk.plan.a.out_ids = out_ids;
         bk.plan.a.out_dists = out_dists;
@@ -200,7 +234,7 @@ int ann_batch_search(ann_batch *bt, const float *queries, int64_t *out_ids, floa
 
 int ann_batch_info(const ann_batch *bt, int32_t *n_buckets, int32_t *k_max) {
     if (!bt) return bfail(ANN_ERR_ARG, "batch is NULL");
-    if (n_buckets) *n_buckets = (int32_t)bt->buckets.size();
+    if (n_buckets) *n_buckets = bt->n_buckets;
     if (k_max) *k_max = bt->kmax;
     return ANN_OK;
 }
