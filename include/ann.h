@@ -124,7 +124,7 @@ typedef struct {
     /* Sync mode only: spread each query over a thread-block cluster of this
      * many CTAs (2, 4 or 8) that share the step's work through distributed
      * shared memory (lower latency per query); 1 = one CTA per query;
-     * 0 = automatic: calls of 1 to 8 queries whose steps gather at least 96
+     * 0 = automatic: calls of 1 to 8 queries whose steps gather at least 192
      * KB of rows (M * R rows) run on clusters of 8 CTAs (4 or
      * 2 when the SMs are fewer than 8 per query) if the search is not
      * persistent, asks for no phase counters, uses visited_mode 0 or 4 and

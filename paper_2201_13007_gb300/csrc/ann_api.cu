@@ -213,16 +213,17 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     if (p->merge_rule == 1 && !(p->patience >= 0.f))
         return fail(ANN_ERR_ARG, "patience must be >= 0 (or INFINITY) with merge_rule 1");
     if (async && M > 32) return fail(ANN_ERR_ARG, "async mode runs one warp per walker: M=%d > 32", M);
-    // cluster = 0, at most 8 queries and steps that gather 96 KB of rows or more: each query on a cluster of 8 CTAs (4,
+    // cluster = 0, at most 8 queries and steps that gather 192 KB of rows or more: each query on a cluster of 8 CTAs (4,
     // 2 if fewer SMs), when the cluster kernel runs the search as asked (sync, not persistent, no phase counters, no
     // neighbour groups, a set-associative visited set); the results are those of one CTA per query. If that plan does
     // not fit, one CTA per query. The lines, us for one query (and for eight), 8 CTAs against one: 96-d BF16 rows, M = 8
-    // (48 KB) 107 / 98 (109 / 98), M = 16 (96 KB) 112 / 116 (124 / 126), M = 32 156 / 167 (181 / 201); 128-d FP32, M = 32
-    // 90 / 110 (101 / 127); 960-d FP8, M = 8 165 / 193 (eight). Above eight queries a cluster gains nothing alone (33
-    // queries, M = 16: 128 / 127) and takes the SMs of calls on other streams (six streams of them: 555 / 248).
+    // (48 KB) 107 / 98 (109 / 98), M = 16 (96 KB) 112 / 116 (124 / 126), M = 32 156 / 167 (181 / 201); 128-d FP32, M = 8
+    // (128 KB) 66 / 64 (83 / 79), M = 32 90 / 110 (101 / 127); 960-d FP8, M = 8 165 / 193 (eight). Above eight queries a
+    // cluster gains nothing alone (33 queries, M = 16: 128 / 127) and takes the SMs of calls on other streams (six
+    // streams of them: 555 / 248).
     if (p->cluster == 0 && nq >= 1 && nq <= 8 && !async && !p->persistent && !p->phase_cycles &&
         (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0 &&
-        (int64_t)M * x.R * x.d_pad * ann::storage_bytes(x.storage) >= (96 << 10)) {
+        (int64_t)M * x.R * x.d_pad * ann::storage_bytes(x.storage) >= (192 << 10)) {
         for (int c = 8; c >= 2; c >>= 1) {
             if ((int64_t)nq * c > sm_count()) continue;
             ann_search_params pc = *p;
@@ -264,10 +265,11 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
             return fail(ANN_ERR_ARG, "threads=%d not in {64,...,1024}", threads);
         if (threads / 32 < M) return fail(ANN_ERR_ARG, "async mode needs threads >= 32*M");
     } else {
-        // clusters: 512 threads for steps of 2,048 slots, 256 for steps of 256 slots or long queues, else 128 (clusters
+        // clusters: 512 threads for steps of 2,048 slots, 256 above 256 slots or for long queues, else 128 (clusters
         // of 8, 512 / 256 / 128 threads, us: 128-d FP32 L = 576, M = 64 138 / 150 / 192, M = 32 172 / 177 / 216; 96-d BF16
-        // L = 192, M = 16 119 / 112 / 124, L = 1024, M = 4 996 / 912 / 934; 960-d FP16 L = 768, M = 16 455 / 422 / 480)
-        if (threads == 0 && !one) threads = slots >= 2048 ? 512 : (slots >= 256 || L >= 384 ? 256 : 128);
+        // L = 192, M = 16 119 / 112 / 124, L = 1024, M = 4 996 / 912 / 934; 960-d FP16 L = 768, M = 16 455 / 422 / 480,
+        // FP8 L = 128, M = 8 - / 151 / 140)
+        if (threads == 0 && !one) threads = slots >= 2048 ? 512 : (slots > 256 || L >= 384 ? 256 : 128);
         if (threads == 0) {
             if (few) {
                 threads = slots * row_bytes >= (384 << 10) || (load <= sms && slots >= 1024) ? 512 : 256;

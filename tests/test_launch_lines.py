@@ -10,7 +10,7 @@ from paper_2201_13007_gb300 import synth  # noqa: E402
 # (queries, L, M) and the automatic (CTAs per query, threads) over 128-d FP32 and BF16 rows (512 and 256 bytes, 32 to a
 # vertex) on a GPU of 152 SMs
 LINES = [
-    ((1, 48, 4), (1, 256), (1, 256)), ((8, 100, 6), (8, 128), (1, 256)), ((8, 100, 12), (8, 256), (8, 256)),
+    ((1, 48, 4), (1, 256), (1, 256)), ((8, 100, 11), (1, 256), (1, 256)), ((8, 100, 12), (8, 256), (1, 256)),
     ((8, 100, 64), (8, 512), (8, 512)), ((9, 100, 64), (1, 512), (1, 512)), ((152, 100, 32), (1, 512), (1, 512)),
     ((153, 100, 32), (1, 512), (1, 256)), ((304, 100, 24), (1, 512), (1, 256)), ((305, 100, 24), (1, 256), (1, 256)),
     ((608, 100, 8), (1, 256), (1, 256)), ((609, 100, 8), (1, 128), (1, 128)), ((609, 100, 32), (1, 256), (1, 256)),
