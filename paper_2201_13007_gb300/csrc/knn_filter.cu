@@ -473,11 +473,15 @@ __global__ void knn_base_rows(const __nv_bfloat16 *__restrict__ x, int64_t n, in
 // that every row is kept whose exact key is among the k smallest. With u =
 // 2^-22, a product sum of d elements in FP32 is off by at most (d + 16) u |q| |x|
 // in any order and with truncated sums, F by at most (d + 32) u (|q| |x| + |x|^2 / 2);
-// keys take two more sums, 8 units in the last place of (|q| + |x|)^2. The
-// k-th F, the k-th key and the key at hand can each be off: three times.
+// keys take two more sums, 8 units in the last place of (|q| + |x|)^2. That
+// holds down to the smallest normal number, 2^-126; below it a product, a sum or
+// a part of the bias (BF16 ends at 2^-133) can lose up to 2^-126 each, 2 d + 64
+// of them at most. The k-th F, the k-th key and the key at hand can each be off:
+// three times. Vectors so short that this second part decides (|x| below 1e-15)
+// all meet the bound, and their blocks are scanned.
 __device__ __forceinline__ float knn_row_margin(float qn, float top, int d) {
     const float q = sqrtf(qn), x = sqrtf(top);
-    return 3.f * ((d + 32) * 2.4e-7f * (2.f * q * x + x * x) + 8.f * 1.2e-7f * (q + x) * (q + x));
+    return 3.f * ((d + 32) * 2.4e-7f * (2.f * q * x + x * x) + 8.f * 1.2e-7f * (q + x) * (q + x) + (d + 32) * 0x1p-125f);
 }
 
 // Per query row of a chunk (padded to whole blocks): its norm, margin, first
