@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(KNT, 1)
                     int32_t *__restrict__ out_ids, float *__restrict__ out_d, const int *__restrict__ only,
                     int *__restrict__ err) {
     if (only && !only[blockIdx.x]) return;
+    if (__syncthreads_or(threadIdx.x == 0 && *static_cast<volatile int *>(err))) return;  // read by one thread: it may change
     constexpr int D = KS * 16;
     constexpr int P = knn_pitch(D);
     constexpr int CPR = D / 8;  // 16-byte chunks per row

@@ -52,7 +52,9 @@ constexpr int FSEG = 32;        // most segments
 // of the byte kPadByte, three times -6.2e32.
 constexpr float kOpen = 1e31f;
 constexpr int kPadByte = 0xF5;
-constexpr uint32_t kSpin = 1u << 20;  // most tries of one wait (each may suspend for up to 20 us)
+// Most tries of one wait; each may suspend for up to 20 us, so a wait that never ends costs 0.33 s at most. The longest
+// that ends, an epilogue in which every value passes, takes some 100 us.
+constexpr uint32_t kWaits = 1u << 14;
 
 // ---------------------------------------------------------------- PTX
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -69,7 +71,7 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // Waits for the phase of the given parity; false if it did not come within
 // the limit, or if another warp of the CTA has given up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *gave_up) {
-    for (uint32_t i = 0; i < kSpin; ++i) {
+    for (uint32_t i = 0; i < kWaits; ++i) {
         uint32_t done;
         asm volatile(
             "{\n.reg .pred p;\n"
@@ -199,8 +201,9 @@ struct FilterArgs {
     uint2 *lists;           // [row][subs][FCAP] of (F, id)
     int32_t *counts;        // [row][subs]
     int *over;              // per 128 query rows: 1 = a list ran over
-    int *err;
+    int *err;               // set to 2 if a wait ran out; a launch that finds it set does nothing
     uint32_t first;         // the segment: base rows first, first + 2^shift, ...
+    int no_loads;           // 1 = load nothing, so that every wait for data runs out (the error path, for tests)
     int shift, subs;
     int tiles, blocks, splits;
 };
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(FTHREADS, 1)
     auto acc_empty = [&](int i) { return bars + 8u * (2 * ST + 6 + i); };
     const uint32_t drained = bars + 8u * (2 * ST + 8);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tail + 8 * (2 * ST + 9));
-    volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 1), *failed = gave_up + 1;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     if (tid == 0) {
@@ -255,6 +258,7 @@ __global__ void __launch_bounds__(FTHREADS, 1)
         }
         mbar_init(drained, 1);
         *gave_up = 0;
+        *failed = *static_cast<volatile int *>(a.err);  // read once: other CTAs of this launch may set it
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid >= 128 && tid < 128 + KBM) {  // the query's side of the bias step: eight elements 1 1 1 0 ..., then eight zeros
@@ -272,10 +276,10 @@ __global__ void __launch_bounds__(FTHREADS, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
-    const int items = a.blocks * a.splits;
+    const int items = *failed ? 0 : a.blocks * a.splits;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (lane == 0 && !a.no_loads) {
             uint32_t nb = 0, ni = 0;  // tiles and items loaded
             bool ok = true;
             for (int it = blockIdx.x; ok && it < items; it += gridDim.x) {
@@ -301,7 +305,8 @@ __global__ void __launch_bounds__(FTHREADS, 1)
                 volatile int never = 0;
                 for (uint32_t i = nb > (uint32_t)ST ? nb - ST : 0; i < nb && !never; ++i)
                     mbar_wait(b_full(i % ST), (i / ST) & 1, &never);
-                for (uint32_t i = ni > 2 ? ni - 2 : 0; i < ni && !never; ++i) mbar_wait(a_full(i & 1), (i >> 1) & 1, &never);
+                for (uint32_t i = ni > 2 ? ni - 2 : 0; i < ni && !never; ++i)
+                    mbar_wait(a_full(i & 1), (i >> 1) & 1, &never);
             }
         }
     } else if (warp == 1) {
@@ -560,7 +565,8 @@ __global__ void __launch_bounds__(256) knn_tighten_kernel(const uint2 *__restric
     for (int i = lane; i < had; i += 32) b[i] = keep[i];
     int n = had;
     for (int s0 = 0; s0 < used; s0 += 32) {
-        const int c = s0 + lane < used ? counts[(size_t)row * subs + s0 + lane] : 0;
+        // (after a wait that ran out, counts and lists may hold anything: nothing here goes by the values of a list)
+        const int c = s0 + lane < used ? min(max(counts[(size_t)row * subs + s0 + lane], 0), FCAP) : 0;
         int end = c;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -644,14 +650,14 @@ __global__ void __launch_bounds__(256)
     knn_finish_kernel(const __nv_bfloat16 *__restrict__ base, const float *__restrict__ bnorm,
                       const __nv_bfloat16 *__restrict__ queries, const float *__restrict__ qnorm, int64_t nq,
                       int64_t self0, int k, const uint2 *__restrict__ kept, const int32_t *__restrict__ kept_n,
-                      int32_t *__restrict__ out_ids, float *__restrict__ out_d) {
+                      int32_t *__restrict__ out_ids, float *__restrict__ out_d, const int *__restrict__ err) {
     constexpr int D = KS * 16;
     __shared__ __align__(16) unsigned long long key_buf[8][FKEEP];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t row = (int64_t)blockIdx.x * 8 + warp;
     if (row >= nq) return;
     unsigned long long *keys = key_buf[warp];
-    const int c = kept_n[row];
+    const int c = *err ? 0 : kept_n[row];  // after a wait that ran out the ids kept may be anything
     const int g = lane >> 2, t = lane & 3;
     uint32_t a[KS][4];
     const uint32_t *q = reinterpret_cast<const uint32_t *>(queries + row * D);
@@ -752,10 +758,10 @@ cudaError_t launch_filter(const RowMaps &q, const RowMaps &x, const FilterArgs &
 template <int KS, bool L2>
 cudaError_t launch_finish(const void *base, const float *norms, const void *q, const float *qnorm, int64_t nq,
                           int64_t self0, int k, const uint2 *kept, const int32_t *kept_n, int32_t *ids, float *dists,
-                          cudaStream_t s) {
+                          const int *err, cudaStream_t s) {
     knn_finish_kernel<KS, L2><<<(unsigned)((nq + 7) / 8), 256, 0, s>>>(
         reinterpret_cast<const __nv_bfloat16 *>(base), norms, reinterpret_cast<const __nv_bfloat16 *>(q), qnorm, nq,
-        self0, k, kept, kept_n, ids, dists);
+        self0, k, kept, kept_n, ids, dists, err);
     return cudaGetLastError();
 }
 
@@ -780,6 +786,7 @@ cudaError_t launch_knn_scan_all(void *ws, const void *base, int64_t n, int d, co
 
 KnnPlan knn_plan(int64_t n, int64_t nq, int sms) {
     KnnPlan p;
+    p.no_loads = 0;
     p.levels = 0;
     while ((n + (int64_t(1) << p.levels) - 1) >> p.levels > FN) ++p.levels;
     // three rounds of 128 query rows per SM in a chunk: a segment's launch is long enough to fill the chip, and the
@@ -861,6 +868,7 @@ cudaError_t launch_knn_bf16(const KnnPlan &p, void *ws, const void *base, int64_
             a.counts = counts;
             a.over = over;
             a.err = err;
+            a.no_loads = p.no_loads;
             a.subs = FEPI / 4 * p.splits;
             a.tiles = (int)((segment_count(n, p.levels, i) + FN - 1) / FN);
             a.blocks = blocks;
@@ -883,8 +891,8 @@ cudaError_t launch_knn_bf16(const KnnPlan &p, void *ws, const void *base, int64_
         float *od = dists + r0 * k;
 #define ANN_KNN_FINISH(KS)                                                                                     \
     case KS:                                                                                                   \
-        e = l2 ? launch_finish<KS, true>(base, norms, q, qnorm, cq, cself, k, kept, kept_n, oi, od, s)         \
-               : launch_finish<KS, false>(base, norms, q, qnorm, cq, cself, k, kept, kept_n, oi, od, s);       \
+        e = l2 ? launch_finish<KS, true>(base, norms, q, qnorm, cq, cself, k, kept, kept_n, oi, od, err, s)    \
+               : launch_finish<KS, false>(base, norms, q, qnorm, cq, cself, k, kept, kept_n, oi, od, err, s);  \
         break;
         switch (d / 16) {
             ANN_KNN_FINISH(2)
