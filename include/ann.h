@@ -257,7 +257,7 @@ int ann_index_group_neighbors(ann_index *index, float hot_fraction, int32_t pref
  * for few queries, one for every 2,048 rows; 1 for many). That is at most 302 MB
  * beside the base rows' part, however many queries there are (3,000 queries
  * over a large base 206 MB, 20,000 187 MB); with no room for it, 4 bytes per
- * base row, and the call is slower. */
+ * base row, and the call is slower. The smallest calls take those 4 bytes. */
 int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, int64_t nq, int64_t self_offset,
                  int32_t metric, int32_t k, int32_t *out_ids, float *out_dists, void *stream);
 

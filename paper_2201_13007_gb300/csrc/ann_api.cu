@@ -589,8 +589,9 @@ int ann_knn_bf16(const void *base, int64_t n, int32_t d, const void *queries, in
     const ann::KnnPlan plan = ann::knn_plan(n, nq, sms);
     unsigned char *ws = nullptr;
     size_t err_at = plan.err;
-    cudaError_t e = cudaMalloc(&ws, plan.bytes);
-    const bool scan = e == cudaErrorMemoryAllocation;  // no room for the filter's lists: 4 bytes a base row will do
+    bool scan = ann::knn_scan_is_faster(n, nq);
+    cudaError_t e = scan ? cudaSuccess : cudaMalloc(&ws, plan.bytes);
+    scan |= e == cudaErrorMemoryAllocation;  // no room for the filter's lists: 4 bytes a base row will do
     if (scan) {
         cudaGetLastError();
         err_at = 0;

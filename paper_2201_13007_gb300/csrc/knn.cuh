@@ -20,8 +20,10 @@ KnnPlan knn_plan(int64_t n, int64_t nq, int sms);
 cudaError_t launch_knn_bf16(const KnnPlan &plan, void *ws, const void *base, int64_t n, int d, const void *queries,
                             int64_t nq, int64_t self0, int metric, int k, int32_t *ids, float *dists, int sms,
                             cudaStream_t stream);
-// The same by the scan kernel alone, for callers without room for the plan's
-// workspace: ws holds knn_scan_bytes(n); its first int is the error word.
+// The same by the scan kernel alone, for small calls (knn_scan_is_faster) and
+// callers without room for the plan's workspace: ws holds knn_scan_bytes(n);
+// its first int is the error word.
+bool knn_scan_is_faster(int64_t n, int64_t nq);
 size_t knn_scan_bytes(int64_t n);
 cudaError_t launch_knn_scan_all(void *ws, const void *base, int64_t n, int d, const void *queries, int64_t nq,
                                 int64_t self0, int metric, int k, int32_t *ids, float *dists, cudaStream_t stream);

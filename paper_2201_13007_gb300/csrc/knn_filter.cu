@@ -784,6 +784,15 @@ cudaError_t launch_knn_scan_all(void *ws, const void *base, int64_t n, int d, co
                            reinterpret_cast<int *>(w), s);
 }
 
+// The filter costs a few launches more than the scan, and an allocation of over 2 MB (640 queries) 125 us. Scan and
+// filter, us, 128-d rows, k = 64 (32-d rows): one query of 64 rows 47 / 62 (38 / 58), of 257 rows 83 / 81 (60 / 76), of
+// 512 rows 93 / 84 (73 / 78), 16 queries of 64 rows 50 / 70 (47 / 58), of 257 rows 96 / 87 (74 / 79), 32 of 64 rows
+// 61 / 70 (50 / 58); 1,000 queries of 64 rows 96 / 183, of 257 rows 219 / 208, 4,000 of 257 rows 224 / 240, of 400 rows
+// 261 / 253; 512 queries of 64 rows 96 / 71.
+bool knn_scan_is_faster(int64_t n, int64_t nq) {
+    return n <= 128 ? nq <= 16 || nq > 640 : n <= 320 && (nq <= 4 || nq > 640);
+}
+
 KnnPlan knn_plan(int64_t n, int64_t nq, int sms) {
     KnnPlan p;
     p.no_loads = 0;
