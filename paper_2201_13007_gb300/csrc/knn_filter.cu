@@ -25,7 +25,7 @@
 // order can make (knn_row_margin), so no row that belongs to a result is
 // dropped. Where a list runs over (many equal distances, a base that defeats
 // the sampling, values that are not finite), the 128 query rows concerned are
-// done again by the scan kernel.
+// done again by the scan kernel; a row given up meets no bound from then on.
 //
 // Measured, all rows against all, k = 64, whole call: 200,000 x 96 in 73.5 ms
 // before and 11.5 ms now (668 TFLOP/s), 20,000 x 128 in 2.93 and 0.94 ms. Of
@@ -606,9 +606,12 @@ __global__ void __launch_bounds__(256) knn_tighten_kernel(const uint2 *__restric
         out += __popc(bal);
     }
     if (lane == 0) {
-        kept_n[row] = min(out, FKEEP);
-        if (last > -kOpen) thr[row] = bound;
-        if (full || out > FKEEP) over[row / KBM] = 1;
+        // No more values of a row that is the scan's: where the norms are far above the distances all of them would
+        // pass, in every segment (20,000 x 96 rows at an offset of 30: 4.67 ms; with none 3.33, the scan alone 2.86)
+        const bool lost = full || out > FKEEP;
+        kept_n[row] = lost ? 0 : out;
+        if (last > -kOpen) thr[row] = lost ? -__int_as_float(0x7F800000) : bound;
+        if (lost) over[row / KBM] = 1;
     }
 }
 
