@@ -126,7 +126,9 @@ typedef struct {
      * shared memory (lower latency per query); 1 = one CTA per query;
      * 0 = automatic: calls of 1 to 8 queries whose steps gather at least 192
      * KB of rows (M * R rows) run on clusters of 8 CTAs (4 or
-     * 2 when the SMs are fewer than 8 per query) if the search is not
+     * 2 when the SMs are fewer than 8 per query), and those with L >= 512 and
+     * rows of at most 512 bytes from 128 KB (rows over 256 bytes from 96 KB)
+     * on clusters of 4, if the search is not
      * persistent, asks for no phase counters, uses visited_mode 0 or 4 and
      * the index has no neighbour groups; otherwise one CTA per query. The
      * results do not depend on the choice. A clustered search is never

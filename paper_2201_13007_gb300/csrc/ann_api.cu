@@ -213,18 +213,26 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
     if (p->merge_rule == 1 && !(p->patience >= 0.f))
         return fail(ANN_ERR_ARG, "patience must be >= 0 (or INFINITY) with merge_rule 1");
     if (async && M > 32) return fail(ANN_ERR_ARG, "async mode runs one warp per walker: M=%d > 32", M);
-    // cluster = 0, at most 8 queries and steps that gather 192 KB of rows or more: each query on a cluster of 8 CTAs (4,
-    // 2 if fewer SMs), when the cluster kernel runs the search as asked (sync, not persistent, no phase counters, no
+    // cluster = 0, at most 8 queries and steps that gather 192 KB of rows or more: each query on a cluster of 8 CTAs (4, 2
+    // if fewer SMs; 4 from 96 or 128 KB with long queues, see below), when the cluster kernel runs the search as asked (sync, not persistent, no phase counters, no
     // neighbour groups, a set-associative visited set); the results are those of one CTA per query. If that plan does
     // not fit, one CTA per query. The lines, us for one query (and for eight), 8 CTAs against one: 96-d BF16 rows, M = 8
     // (48 KB) 107 / 98 (109 / 98), M = 16 (96 KB) 112 / 116 (124 / 126), M = 32 156 / 167 (181 / 201); 128-d FP32, M = 8
     // (128 KB) 66 / 64 (83 / 79), M = 32 90 / 110 (101 / 127); 960-d FP8, M = 8 165 / 193 (eight). Above eight queries a
     // cluster gains nothing alone (33 queries, M = 16: 128 / 127) and takes the SMs of calls on other streams (six
     // streams of them: 555 / 248).
+    // Long queues (L >= 512) of rows up to 512 bytes: 4 CTAs, from 96 KB on for rows over 256 bytes and from 128 KB for
+    // shorter ones. us for one and for eight queries, 4 CTAs against one (8): 128-d FP32, M = 6 (96 KB), L = 1024 793, 908 /
+    // 836, 1031 (777, 866); M = 8, L = 576 377, 426 / 397, 447 (365, 397); M = 11, L = 576 307, 343 / 347, 391 (293, 319);
+    // 96-d BF16, M = 16 (96 KB), L = 1024 331, 400 / 326, 408 (323, 388), M = 31 228, 295 / 251, 343 (221, 277). 8 CTAs are
+    // faster alone, but six streams of eight queries then take 1,144 us (FP32, L = 1024, M = 8) against 905 with 4 CTAs
+    // and 900 with one. 960-d FP8 rows lose alone (L = 1024, M = 6, one query 1,108 / 994).
+    const int64_t step_row = (int64_t)x.d_pad * ann::storage_bytes(x.storage), step_bytes = (int64_t)M * x.R * step_row;
+    const int64_t from4 = step_row > 256 ? 96 << 10 : 128 << 10;
+    const int auto_cluster = step_bytes >= (192 << 10) ? 8 : L >= 512 && step_row <= 512 && step_bytes >= from4 ? 4 : 1;
     if (p->cluster == 0 && nq >= 1 && nq <= 8 && !async && !p->persistent && !p->phase_cycles &&
-        (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0 &&
-        (int64_t)M * x.R * x.d_pad * ann::storage_bytes(x.storage) >= (192 << 10)) {
-        for (int c = 8; c >= 2; c >>= 1) {
+        (p->visited_mode == 0 || p->visited_mode == 4) && x.n_hot == 0) {
+        for (int c = auto_cluster; c >= 2; c >>= 1) {
             if ((int64_t)nq * c > sm_count()) continue;
             ann_search_params pc = *p;
             pc.cluster = c;
