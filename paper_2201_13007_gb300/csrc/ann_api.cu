@@ -342,8 +342,12 @@ int plan_search(const ann_index *index, const float *queries, int64_t nq, int32_
                     break;
                 }
             while (vmode == 4 && ways_for(hb) < 2) ++hb;  // more sets leave more bits per tag
-        } else if (vmode == 4) {  // 2^13 sets hold 24,576 tags in 32 KB; 2^14 for clusters' long queues or heavy steps
-            hb = !one && heavy ? 14 : 13;
+        } else if (vmode == 4) {
+            // 2^13 sets hold 24,576 tags in 32 KB; 2^14 for clusters' long queues or heavy steps, and for one query an SM
+            // whose vertices pass that number within few steps and whose repeated distances are long (L = 2048, M = 64, us,
+            // 2^14 / 2^13: 128-d FP32 rows, 33 queries 623 / 902, six streams of 152 2,991 / 3,361; L = 1536 460 / 487, but
+            // 2,329 / 1,952, as fewer reside, and M = 32 754 / 591; 96-d BF16, L = 2048 416 / 489, but 2,051 / 1,676)
+            hb = (one ? load <= sms && L > 1536 && slots >= 2048 && row_bytes > 256 : heavy) ? 14 : 13;
             while (ways_for(hb) < 2) ++hb;
         } else {
             hb = heavy ? 14 : (slots >= 1024 ? 13 : 12);
