@@ -345,8 +345,8 @@ int ann_search_host_noalloc(const ann_index *index, const float *queries, int64_
  * paper, which runs one query at a time). Queries are grouped into buckets
  * by L; each bucket is one persistent grid, sized for the largest L and M of
  * its queries, that pulls them longest-first from a device work list (two
- * grids, by the slots M * R of a step, in batches of more than 32 queries
- * per SM, unless a launch config is given). The
+ * grids, by the slots M * R of a step, in synchronous batches of more than
+ * 32 queries per SM, unless the bucket's or the params' threads are given). The
  * buckets run concurrently on the plan's own streams, forked from and joined
  * back into the caller's stream, so a whole ann_batch_search can be captured
  * into a CUDA graph (it allocates nothing and never synchronises). */

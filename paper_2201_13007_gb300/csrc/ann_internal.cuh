@@ -168,7 +168,8 @@ void set_error(const char *msg);
 cudaError_t ensure_dyn_smem(const void *kernel, int smem);
 
 // ann_api.cu: argument checks and launch configuration of one search. together: how many queries run at the same time,
-// which the automatic launch shape goes by (0: the nq of this search; a batch gives the queries of all its launches)
+// which the automatic launch shape goes by (0: the nq of this search; a batch whose buckets run as two launches gives the
+// queries of all of them)
 struct Plan {
     SearchArgs a;
     int threads;

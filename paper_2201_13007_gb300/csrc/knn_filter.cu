@@ -28,8 +28,8 @@
 // done again by the scan kernel; a row given up meets no bound from then on.
 //
 // Measured, all rows against all, k = 64, whole call: 200,000 x 96 in 73.5 ms
-// before and 11.5 ms now (668 TFLOP/s), 20,000 x 128 in 2.93 and 0.94 ms. Of
-// the 11.5 ms the filter takes 8.7, the tightens 1.7, the finish 0.8.
+// before and 11.6 ms now (662 TFLOP/s), 20,000 x 128 in 2.93 and 0.92 ms. Of
+// the 11.6 ms the filter takes 8.7, the tightens 1.8, the finish 0.8.
 #include <cuda.h>
 
 #include <algorithm>

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 2) cluster_search_kernel(c
     }
     for (;;) {
         const int par = step & 1;
-        // --- select (every CTA, identical): the first Mcur unchecked entries, all warps scanning
+        // --- select (every CTA, identical): the first Mcur unchecked entries, warp 0 scanning
         const int found = select_step(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, &ctl.sel_found, tid);
         ANN_CPHASE(0)
         const int nact = found < Mcur ? found : Mcur;

@@ -309,16 +309,6 @@ __device__ __forceinline__ void compute_keys_teams_m(const void *rows, const flo
     }
 }
 
-template <int STORE, int NT, int G = 2>
-__device__ __forceinline__ void compute_keys_teams(const void *rows, const float *scales, int row_elems, int metric,
-                                                   const float *qv, const entry_t *cand, int nc, int lts,
-                                                   entry_t limit, entry_t *out, int *out_n) {
-    if (metric == ANN_METRIC_L2)
-        compute_keys_teams_m<STORE, NT, true, G>(rows, scales, row_elems, qv, cand, nc, lts, limit, out, out_n);
-    else
-        compute_keys_teams_m<STORE, NT, false, G>(rows, scales, row_elems, qv, cand, nc, lts, limit, out, out_n);
-}
-
 // ------------------------------------------------------------- visited set
 // Open addressing over 2^bits uint32 slots (kEmptySlot = free), linear
 // probing. Returns 1 if id was inserted now, 0 if it was already present,
@@ -566,8 +556,8 @@ __device__ __forceinline__ entry_t warp_sort32(entry_t v) {
     return v;
 }
 
-// Ascending sort of in[0..n), 32 < n <= NT, into out[0..n) (disjoint from
-// in). Warp w sorts the run in[32w, 32w + 32) in registers and writes it
+// Ascending sort of in[0..n), 1 <= n <= NT, into out[0..n) (disjoint from
+// in, which holds whole runs of 32). Warp w sorts the run in[32w, 32w + 32) in registers and writes it
 // back; each element's rank is then its lane plus, for every other run, the
 // entries of that run below it (runs after its own) or not above it (runs
 // before its own), by a branch-free binary search. Equal entries thus keep
@@ -1264,7 +1254,7 @@ __device__ __forceinline__ void move_queue(const entry_t *Q, int qlen, const int
     }
 }
 
-// The merge for few survivors (ns <= NT, one a thread), which most steps
+// The merge for few survivors (ns <= min(NT, 128), one a thread), which most steps
 // have (of the 25 steps of a query at L = 576, M = 32: 13 with 32 or fewer, 18
 // with 128 or fewer): nothing is sorted. A survivor's place in the new queue is the number of
 // queued entries below it (a binary search) plus the number of survivors below
@@ -1331,7 +1321,7 @@ __device__ __forceinline__ int merge_by_rank(const entry_t *Q, int qlen, entry_t
     }
 }
 
-// Sorts in[0..n) by (key, id), n > 1 (one a thread: warp runs plus binary-search
+// Sorts in[0..n) by (key, id), n > 0 (one a thread: warp runs plus binary-search
 // ranks into `scratch`; above that warp runs merged pairwise between in and
 // `scratch`), and, with `unsafe`, drops entries whose id is queued in Q[0..qlen)
 // or repeated (counted in *dropped). Returns the sorted array and in *n what it
@@ -1383,7 +1373,7 @@ __device__ __forceinline__ entry_t *sort_dedupe(const entry_t *Q, int qlen, entr
 }
 
 // The ns (> 0) survivors in surv, in no order, are merged into the sorted
-// queue Q[0..qlen): up to 128 (256 in CTAs of 512 threads) by rank
+// queue Q[0..qlen): up to 128 (64 in CTAs of 64 threads) by rank
 // (merge_by_rank), more sorted first (one a
 // thread: warp runs plus binary-search ranks into `scratch`; above that warp
 // runs merged pairwise between surv and `scratch`) and merged by merge path.

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(NT, 65536 / (NT * 64)) sync_search_kernel(cons
                 __syncthreads();
             }
             const int par = step & 1;
-            // --- select: the first Mcur unchecked entries (rank order) of the stable queue, all warps
+            // --- select: the first Mcur unchecked entries (rank order) of the stable queue, warp 0
             // scanning from first_un (entries before it are all checked)
             const int found = select_step(Q, qlen, ctl.first_un, Mcur, sel_id, sel_pos, &ctl.sel_found, tid);
             const int nact = found < Mcur ? found : Mcur;
